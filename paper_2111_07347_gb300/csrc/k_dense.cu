@@ -35,6 +35,7 @@
 #include <math.h>
 
 #include "tm_internal.h"
+#include "tm_tcgen05.h"
 
 namespace tmgb {
 namespace {
@@ -52,112 +53,11 @@ constexpr int kEpiWarp0 = 4;
 constexpr int kEpiWarps = 8;               // two per TMEM lane quadrant, each half of the shift columns
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kThreads = (kEpiWarp0 + kEpiWarps) * 32;
-constexpr unsigned long long kTimeoutNs = 1000000000ull;   // 1 s per wait
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t globaltimer() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t addr, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(addr), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t addr) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(addr) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t addr, uint32_t bytes) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(addr),
-                 "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t addr, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait; false on timeout or when another role has aborted.
-__device__ bool mbar_wait(uint32_t addr, uint32_t parity, volatile int* abort_flag) {
-    uint64_t t0 = 0;
-    for (uint32_t it = 0;; ++it) {
-        if (mbar_try(addr, parity)) return true;
-        if ((it & 255u) == 255u) {
-            if (*abort_flag) return false;
-            const uint64_t t = globaltimer();
-            if (t0 == 0) t0 = t;
-            else if (t - t0 > kTimeoutNs) return false;
-        }
-    }
-}
-
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void named_bar(int id, int count) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
-// 4-D tiled TMA load (coordinates innermost first) completing on an mbarrier.
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            uint32_t mbar) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-        "[%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-        "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(mbar)
-        : "memory");
-}
-
-// Shared-memory matrix descriptors (128-byte swizzle).  K-major: rows of 64 K-elements, 8-row
-// groups 1024 B apart.  MN-major: rows of 64 MN-elements (one per K index), 8 K-rows 1024 B
-// apart (stride dimension), 64-element MN blocks `mn_stride` bytes apart (leading dimension).
-__device__ __forceinline__ uint64_t sdesc_kmajor(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-__device__ __forceinline__ uint64_t sdesc_mnmajor(uint32_t saddr, uint32_t mn_stride) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)((mn_stride >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
 
 // Instruction descriptor: kind::f16, A = B = BF16, D = F32, A MN-major (bit 15), B K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16_amn(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(N >> 3) << 17) |
            ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-                 : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
@@ -279,7 +179,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_kernel(const __grid_constan
                     for (int ks = 0; ks < kChunk / 16; ++ks) {
                         const uint64_t a = sdesc_mnmajor(ring0 + slot * kSlotBytes + ks * 2048, kBoxBytes);
                         const uint64_t b = sdesc_kmajor(basis0 + ch * kBasisChunkBytes + ks * 32);
-                        mma_bf16(d, a, b, idesc, (ch % (kChunks / 2) == 0 && ks == 0) ? 0u : 1u);
+                        mma_f16(d, a, b, idesc, (ch % (kChunks / 2) == 0 && ks == 0) ? 0u : 1u);
                     }
                     mma_commit(bar_empty0 + 8 * slot);
                     last_bar = bar_empty0 + 8 * slot;

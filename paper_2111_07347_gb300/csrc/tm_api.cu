@@ -70,6 +70,7 @@ struct Library {
     int64_t n_sym = 0, macs = 0;
     int max_spots = 0;
     int nonneg = 1;                // every intensity >= 0
+    bool unit = false;             // loaded with TM_LIB_UNIT_INTENSITY
     // host copies (exported for tests)
     std::vector<int64_t> off;
     std::vector<int32_t> r, t, order;
@@ -98,6 +99,11 @@ struct Library {
     int32_t* d_rowmap = nullptr;   // [n_r] radius -> row among the distinct radii (-1: none)
     int R = 0, K_pad = 0;
     size_t that_bytes = 0;
+    // templates of the tensor-core bounds (k_bound.cu), built on first use: [K][pitch] FP16
+    tmgb::BoundShape bshape;
+    void* d_bound = nullptr;
+    int4* d_border = nullptr;      // [32 words] the templates in the bounds' order, fewest spots first
+    size_t bound_bytes = 0;
 };
 
 struct Buffer {
@@ -189,7 +195,7 @@ struct tm_ctx {
     unsigned long long* d_work = nullptr;   // sparse multiply-adds executed while profiling
     std::map<int, SpectralTables> spectral;
     cublasHandle_t cublas = nullptr;                     // stage A of the tensor-core path
-    PFN_cuTensorMapEncodeTiled_v12000 encode_tiled = nullptr;
+    PFN_cuTensorMapEncodeTiled_v12000 encode_tiled = nullptr;   // tensor maps of the tensor-core kernels
     std::map<std::string, RadiusMap> radius_maps;
     // CUDA graphs of whole-path calls (TM_INDEX_GRAPH)
     struct GraphEntry {
@@ -371,6 +377,7 @@ int prepare_library(const tm_library_desc* d, Library* L, Prepared* P) {
     if (n_r >= 8192 || n_theta >= 2048)
         return fail(TM_ERR_UNSUPPORTED, "tm_load_library: polar grid %dx%d too large for the sparse layout", n_r, n_theta);
     L->K0 = K0;
+    L->unit = unit;
     L->mirror = (d->flags & TM_LIB_MIRROR) ? 1 : 0;
     L->K = K0 * (L->mirror ? 2 : 1);
     L->n_r = n_r;
@@ -611,10 +618,11 @@ int build_library(tm_ctx* ctx, const tm_library_desc* d, Library* L) {
 void free_library(tm_ctx* ctx, Library* L) {
     void* ps[] = {L->d_off,    L->d_spot,  L->d_spot2, L->d_meta,  L->d_norm,   L->d_nshift, L->d_radial,
                   L->d_rnorm,  L->d_rt,    L->d_radii, L->d_bspot, L->d_that,   L->d_rowmap,
-                  L->d_smeta,  L->d_sperm, L->d_ellw,  L->d_ell};
+                  L->d_smeta,  L->d_sperm, L->d_ellw,  L->d_ell,  L->d_bound,
+                  L->d_border};
     for (void* p : ps)
         if (p) cudaFree(p);
-    ctx->used -= std::min(ctx->used, L->bytes + L->that_bytes);
+    ctx->used -= std::min(ctx->used, L->bytes + L->that_bytes + L->bound_bytes);
 }
 
 tmgb::SparseLib sparse_view(const Library* L) {
@@ -829,9 +837,65 @@ int ensure_spectra(tm_ctx* ctx, Library* L, const SpectralTables& spec, cudaStre
     return TM_OK;
 }
 
-// Tensor map of G [192][nb][2][K_pad] BF16 for stage B: 4-D (k, c, p, j), boxes of
-// 64 templates x 2 x 1 pattern x 32 slots, 128-byte swizzle, zero fill past K.
-int g_tensor_map(tm_ctx* ctx, void* g, int K, int K_pad, int64_t nb, CUtensorMap* out) {
+// Whether the library has the templates of the tensor-core bounds, built on the device the first
+// time it is asked (the call waits for the build, so that work on other streams can use them as
+// soon as it returns).  Not for libraries with negative intensities or more radii than the
+// contraction takes, nor while their memory is not to be had (the budget; a stream that is
+// being captured): such calls bound and score in the sparse kernel.
+bool ensure_bounds(tm_ctx* ctx, Library* L, cudaStream_t st) {
+    if (L->d_bound) return true;
+    const int n_rad = (int)std::max<size_t>(1, L->radii.size());
+    // finer windows where templates of like weights compete: unit intensities, or many spots
+    const bool fine = L->unit || (int64_t)L->r.size() >= 20 * L->K;
+    if (!L->nonneg || !tmgb::bound_shape(n_rad, L->n_theta, fine, &L->bshape)) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (ctx->capturing || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    // the order of the bounds: by spot count, fewest first, ties by index
+    std::vector<int32_t> perm(L->K);
+    for (int64_t k = 0; k < L->K; ++k) perm[k] = (int32_t)k;
+    std::stable_sort(perm.begin(), perm.end(),
+                     [&](int32_t a, int32_t b) { return L->off[a + 1] - L->off[a] < L->off[b + 1] - L->off[b]; });
+    std::vector<int4> order((L->K + 31) / 32 * 32, make_int4(0, 0, 0, -1));
+    for (int64_t j = 0; j < L->K; ++j) {
+        const int32_t k = perm[j];
+        int32_t nb;
+        memcpy(&nb, &L->norm[k], 4);
+        order[j] = make_int4((int32_t)L->off[k],
+                             (int32_t)((L->off[k + 1] - L->off[k]) | ((int64_t)(L->n_theta / L->order[k]) << 16)), nb, k);
+    }
+    const size_t bytes = (size_t)L->K * L->bshape.pitch * 2, ob = order.size() * sizeof(int4);
+    void *b = nullptr, *o = nullptr;
+    const std::string err = g_err;
+    if (dev_alloc(ctx, &b, bytes, "library bound templates")) {
+        g_err = err;
+        return false;
+    }
+    if (dev_alloc(ctx, &o, ob, "library bound order")) {
+        g_err = err;
+        dev_free(ctx, b, bytes);
+        return false;
+    }
+    cudaError_t e = cudaMemcpyAsync(o, order.data(), ob, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+        e = tmgb::launch_bound_templates(L->d_meta, (const int4*)o, L->d_spot, (int)L->K, L->n_theta, n_rad, L->bshape,
+                                         b, st);
+    const cudaError_t e2 = cudaStreamSynchronize(st);
+    if (e != cudaSuccess || e2 != cudaSuccess) {
+        cudaGetLastError();
+        dev_free(ctx, b, bytes);
+        dev_free(ctx, o, ob);
+        return false;
+    }
+    L->d_bound = b;
+    L->d_border = (int4*)o;
+    L->bound_bytes = bytes + ob;
+    return true;
+}
+
+int tensor_map_encoder(tm_ctx* ctx) {
     if (!ctx->encode_tiled) {
         void* fn = nullptr;
         cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
@@ -842,6 +906,30 @@ int g_tensor_map(tm_ctx* ctx, void* g, int K, int K_pad, int64_t nb, CUtensorMap
         }
         ctx->encode_tiled = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     }
+    return TM_OK;
+}
+
+// Tensor map of one operand of the bounds' contraction: [rows][pitch] FP16, boxes of 64 entries x
+// `box_rows` rows, 128-byte swizzle, zero fill past the ends.
+int bound_tensor_map(tm_ctx* ctx, void* base, int64_t rows, int pitch, int box_rows, CUtensorMap* out) {
+    const int rc = tensor_map_encoder(ctx);
+    if (rc) return rc;
+    const cuuint64_t dims[2] = {(cuuint64_t)pitch, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)pitch * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+    const cuuint32_t es[2] = {1, 1};
+    const CUresult r = ctx->encode_tiled(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, base, dims, strides, box, es,
+                                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(TM_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
+    return TM_OK;
+}
+
+// Tensor map of G [192][nb][2][K_pad] BF16 for stage B: 4-D (k, c, p, j), boxes of
+// 64 templates x 2 x 1 pattern x 32 slots, 128-byte swizzle, zero fill past K.
+int g_tensor_map(tm_ctx* ctx, void* g, int K, int K_pad, int64_t nb, CUtensorMap* out) {
+    const int rc = tensor_map_encoder(ctx);
+    if (rc) return rc;
     const cuuint64_t dims[4] = {(cuuint64_t)K, 2, (cuuint64_t)nb, (cuuint64_t)tmgb::dense_slots()};
     const cuuint64_t strides[3] = {(cuuint64_t)K_pad * 2, (cuuint64_t)K_pad * 4, (cuuint64_t)nb * K_pad * 4};
     const cuuint32_t box[4] = {64, 2, 1, 32};
@@ -1703,8 +1791,33 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
     int keep[TM_MAX_LIBS];
     for (int i = 0; i < n_libs; ++i) keep[i] = keep_count(params->prefilter_fraction, libs[i]->K);
 
+    // FP32 path: bounds of every template on the tensor cores, then the exact scores of the few
+    // templates they leave (k_bound.cu, k_score.cu), where every library has them; else the sparse
+    // kernel bounds and scores in one.  BF16 path: the candidates are scored by the score kernel.
+    // A library of less than 512 templates is scored whole: the bounds' two launches and their
+    // latency cost more than the scores they would save (300 templates of 24 spots, 256 patterns:
+    // 137 us with bounds, 83 us without).
+    bool bounds = !bf16, scores = true;
+    bool whole[TM_MAX_LIBS];
+    for (int i = 0; i < n_libs; ++i) {
+        scores = scores && tmgb::score_supported((int)std::max<size_t>(1, libs[i]->radii.size()), n_theta, N);
+        whole[i] = libs[i]->K < 512;
+        bounds = bounds && scores && (whole[i] || ensure_bounds(ctx, libs[i], st));
+    }
+
     // chunk size from a per-pattern workspace estimate (<= 4 GiB of workspace)
     size_t per = (size_t)n_r * n_theta * 4 + 4 + (size_t)n_r * 4 + 4;
+    size_t w_per = 0, u_per = 0, wmax_per = 0;              // bounds: bytes per pattern, one library at a time
+    if (bounds) {
+        for (int i = 0; i < n_libs; ++i) {
+            if (whole[i]) continue;
+            const size_t words = (size_t)((libs[i]->K + 31) / 32);
+            w_per = std::max(w_per, (size_t)libs[i]->bshape.nw * libs[i]->bshape.pitch * 2);
+            u_per = std::max(u_per, words * 64);
+            wmax_per = std::max(wmax_per, words * 2);
+        }
+        per += w_per + u_per + wmax_per;
+    }
     for (int i = 0; i < n_libs; ++i)
         if (pre || bf16) per += (size_t)libs[i]->K * 4 + ((libs[i]->K + 31) / 32) * 4;
     size_t cap = (size_t)4 << 30;
@@ -1729,10 +1842,17 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
     __half* seed_qub = nullptr;
     const int seed_ctas = tmgb::sparse_max_ctas(sms);
     const size_t seed_slots = (size_t)seed_ctas * tmgb::kSparseTile;   // one per pattern of a CTA's tile
-    if (!rc) rc = workspace(ctx, st, "seed_bits", seed_slots * max_words * 4, (void**)&seed_bits);
-    if (!rc) rc = workspace(ctx, st, "seed_qub", seed_slots * max_words * 32 * 2, (void**)&seed_qub);
+    const bool seeds = !bounds && !(bf16 && scores);
+    if (!rc && seeds) rc = workspace(ctx, st, "seed_bits", seed_slots * max_words * 4, (void**)&seed_bits);
+    if (!rc && seeds) rc = workspace(ctx, st, "seed_qub", seed_slots * max_words * 32 * 2, (void**)&seed_qub);
     int32_t* seed_cand = nullptr;
-    if (!rc) rc = workspace(ctx, st, "seed_cand", (size_t)seed_ctas * max_words * 32 * 4, (void**)&seed_cand);
+    if (!rc && seeds)
+        rc = workspace(ctx, st, "seed_cand", (size_t)seed_ctas * max_words * 32 * 4, (void**)&seed_cand);
+    void* bw = nullptr;                                      // window columns, bounds, word maxima
+    unsigned short *bu = nullptr, *bmax = nullptr;
+    if (!rc && bounds) rc = workspace(ctx, st, "bound_w", (size_t)chunk * w_per, &bw);
+    if (!rc && bounds) rc = workspace(ctx, st, "bound_u", (size_t)chunk * u_per, (void**)&bu);
+    if (!rc && bounds) rc = workspace(ctx, st, "bound_max", (size_t)chunk * wmax_per, (void**)&bmax);
     TensorBuffers tb;
     if (!rc && bf16) rc = tensor_buffers(ctx, st, tp, std::min<int64_t>(tp.nb, chunk), &tb);
     if (rc) return rc;
@@ -1792,6 +1912,57 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
                     ++launches;
                 }
             }
+            // one library's scores and top N: behind its bounds (kernels counted in `launches`), or of
+            // the candidates in its mask
+            auto score_library = [&](int i) -> int {
+                const Library* L = libs[i];
+                const int n_rad = (int)std::max<size_t>(1, L->radii.size());
+                tmgb::ScoreCall sc{};
+                sc.polar = polar;
+                sc.pnorm = pnorm;
+                sc.n = m;
+                sc.n_r = n_r;
+                sc.n_theta = n_theta;
+                sc.lib = sparse_view(L);
+                sc.mask = pre || bf16 ? mask[i] : nullptr;
+                if (bounds && !whole[i]) {
+                    const tmgb::BoundShape& bs = L->bshape;
+                    CUtensorMap amap, bmap;
+                    int rc2 = bound_tensor_map(ctx, L->d_bound, L->K, bs.pitch, tmgb::bound_box_rows(true), &amap);
+                    if (!rc2)
+                        rc2 = bound_tensor_map(ctx, bw, m * bs.nw, bs.pitch, tmgb::bound_box_rows(false), &bmap);
+                    if (rc2) return rc2;
+                    TM_CUDA(tmgb::launch_bound_windows(polar, pnorm, m, n_r, n_theta, L->d_radii, n_rad, bs, bw, pcount,
+                                                       st),
+                            "tm_index_patterns: bound windows");
+                    tmgb::BoundCall bc{};
+                    bc.n = m;
+                    bc.K = (int)L->K;
+                    bc.words = sc.lib.words;
+                    bc.kd = bs.kd;
+                    bc.u = bu;
+                    bc.wmax = bmax;
+                    bc.error = ctx->d_error;
+                    TM_CUDA(tmgb::launch_bound(&amap, &bmap, bc, bs.nw, sms, st), "tm_index_patterns: bounds");
+                    sc.order = L->d_border;
+                    sc.u = bu;
+                    sc.wmax = bmax;
+                    sc.seeds = bs.nw == 12 ? 64 : 32;
+                    launches += 2;
+                } else {
+                    TM_CUDA(cudaMemsetAsync(pcount, 0, sizeof(int), st), "tm_index_patterns: counter");
+                }
+                sc.hits = out_dev + (size_t)i * lib_stride + (size_t)c0 * N;
+                sc.top_n = N;
+                sc.counter = pcount;
+                sc.work = ctx->profiling ? ctx->d_work : nullptr;
+                sc.bulk = n_theta % 4 == 0 && ((uintptr_t)polar & 15) == 0;
+                sc.error = ctx->d_error;
+                sc.test_stall = (params->reserved & TM_INDEX_TEST_STALL) ? 1 : 0;
+                TM_CUDA(tmgb::launch_score(sc, sms, st), "tm_index_patterns: scores");
+                ++launches;
+                return TM_OK;
+            };
             tmgb::SparseCall c{};
             c.polar = polar;
             c.pnorm = pnorm;
@@ -1838,9 +2009,15 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
                 }
                 {
                     StageTimer tmr(ctx, TM_STAGE_RESCORE, st);
-                    TM_CUDA(tmgb::launch_sparse(c, sms, st), "tm_index_patterns: rescore");
+                    for (int i = 0; scores && i < n_libs; ++i) {
+                        const int rc3 = score_library(i);
+                        if (rc3) return rc3;
+                    }
+                    if (!scores) {
+                        TM_CUDA(tmgb::launch_sparse(c, sms, st), "tm_index_patterns: rescore");
+                        ++launches;
+                    }
                 }
-                ++launches;
                 for (int i = 0; i < n_libs; ++i) {
                     corr += m * ((int64_t)keep[i] + std::min<int64_t>(kc, keep[i])) * n_theta;
                     scored += m * std::min<int64_t>(kc, keep[i]);
@@ -1848,9 +2025,15 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
             } else {
                 {
                     StageTimer tmr(ctx, TM_STAGE_SPARSE, st);
-                    TM_CUDA(tmgb::launch_sparse(c, sms, st), "tm_index_patterns: sparse");
+                    for (int i = 0; bounds && i < n_libs; ++i) {
+                        const int rc2 = score_library(i);
+                        if (rc2) return rc2;
+                    }
+                    if (!bounds) {
+                        TM_CUDA(tmgb::launch_sparse(c, sms, st), "tm_index_patterns: sparse");
+                        ++launches;
+                    }
                 }
-                ++launches;
                 for (int i = 0; i < n_libs; ++i) {
                     corr += m * (int64_t)keep[i] * n_theta;
                     scored += m * keep[i];

@@ -212,6 +212,60 @@ int sparse_pitch(int n_theta, int layout);
 int sparse_rows(int n_rad, int layout);
 cudaError_t launch_sparse(const SparseCall& c, int num_sms, cudaStream_t st);
 
+// ------------------------------------------------------------------ bounds on the tensor cores
+// Upper bounds U[p][k] of the correlation index (k_bound.cu): the azimuth in `pieces` pieces, nch
+// chunks of columns and nw windows of shifts (both runs of pieces); kd = n_rad nch + 1 entries of
+// the contraction, rows of both operands `pitch` halves apart.
+struct BoundShape {
+    int nch = 0, nw = 0, pieces = 0, kd = 0, pitch = 0;
+};
+// The shape for a library of n_rad rows (false: the bounds are not available for it): the finest
+// chunks whose contraction fits 512 entries.
+bool bound_shape(int n_rad, int n_theta, bool fine, BoundShape* out);
+// B [K][pitch] FP16: row j from the template order[j].w.
+cudaError_t launch_bound_templates(const int4* meta, const int4* order, const int2* spot, int K, int n_theta, int n_rad,
+                                   const BoundShape& s, void* out, cudaStream_t st);
+// W [n nw][pitch] FP16 from the polar rows; zeroes *counter (nullable) for the kernels that follow.
+cudaError_t launch_bound_windows(const float* polar, const float* pnorm, int64_t n, int n_r, int n_theta,
+                                 const int32_t* radii, int n_rad, const BoundShape& s, void* w, int* counter,
+                                 cudaStream_t st);
+struct BoundCall {
+    int64_t n;                 // patterns
+    int K, words, kd;
+    unsigned short* u;         // [n][32 words] FP16 as order-preserving keys
+    unsigned short* wmax;      // [n][words] keys: the largest of each 32 templates
+    unsigned* error;           // device word: bit 8 = a bounded wait timed out
+    int stages;                // set by launch_bound
+};
+int bound_box_rows(bool templates);        // rows of the tensor maps' boxes (64 halves wide, 128-byte swizzle)
+cudaError_t launch_bound(const void* amap, const void* bmap, const BoundCall& c, int nw, int num_sms, cudaStream_t st);
+
+// Exact scores of the templates the bounds leave (k_score.cu), or of the templates of a mask, and
+// the top-N, for one library.
+struct ScoreCall {
+    const float* polar;        // [n][n_r][n_theta]
+    const float* pnorm;        // [n]
+    int64_t n;
+    int n_r, n_theta, pitch;   // pitch: set by launch_score (layout row pitch)
+    SparseLib lib;
+    const uint32_t* mask;      // [n][words] templates that take part, or null (all)
+    const int4* order;         // [32 words] {first spot, spots | shifts << 16, norm bits, template} of
+                               // the bounds' positions (template -1: padding)
+    const unsigned short* u;   // [n][32 words] upper bounds by position (keys), or null: every
+                               // template of the mask is scored
+    const unsigned short* wmax;   // [n][words] the bounds' maxima per word
+    int seeds;                 // templates scored first (with bounds): 32 or 64
+    tm_hit* hits;              // [n][top_n]
+    int top_n;
+    int* counter;              // device int, 0 at launch
+    unsigned long long* work;  // nullable: += multiply-adds executed
+    int bulk;                  // as SparseCall
+    unsigned* error;
+    int test_stall;
+};
+bool score_supported(int n_rad, int n_theta, int top_n);
+cudaError_t launch_score(const ScoreCall& c, int num_sms, cudaStream_t st);
+
 // ------------------------------------------------------------------ BF16 tensor-core path
 // Frequency slots of the angular spectra: slot j < 96 holds m = 2 j, slot j >= 96 holds
 // m = 2 (j - 96) + 1 (even frequencies first, for the radix-2 split of stage B); slots whose
