@@ -47,6 +47,50 @@ __global__ void find_centres_kernel(const T* __restrict__ frames, int64_t n, int
     out[p] = make_float2((float)cx, (float)cy);
 }
 
+// u16 frames, one warp per pattern: the sums are of integers below 2^53 (the caller sees to it), so
+// they are exact in any order and equal the serial sums above; every pixel's test and the divisions
+// are the same operations.  A thread per pattern runs the whole disc as one chain of FP64 additions:
+// 168 us for a few patterns and 191 us for 4096, a warp per pattern 16 and 55 us.
+__global__ void __launch_bounds__(128)
+find_centres_u16_kernel(const uint16_t* __restrict__ frames, int64_t n, int H, int W, double cx0, double cy0,
+                        double radius, int iterations, float2* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const int64_t p = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (p >= n) return;
+    const uint16_t* f = frames + (size_t)p * H * W;
+    const double r2 = __dmul_rn(radius, radius);
+    double cx = cx0, cy = cy0;
+    for (int it = 0; it < iterations; ++it) {
+        const int y_lo = max(0, (int)ceil(__dsub_rn(cy, radius)));
+        const int y_hi = min(H - 1, (int)floor(__dadd_rn(cy, radius)));
+        const int x_lo = max(0, (int)ceil(__dsub_rn(cx, radius)));
+        const int x_hi = min(W - 1, (int)floor(__dadd_rn(cx, radius)));
+        const int w = x_hi - x_lo + 1, h = y_hi - y_lo + 1;
+        unsigned long long s0 = 0, sx = 0, sy = 0;
+        for (int i = lane; w > 0 && h > 0 && i < w * h; i += 32) {
+            const int y = y_lo + i / w, x = x_lo + i % w;
+            const unsigned v = __ldg(f + (size_t)y * W + x);
+            const double dy = __dsub_rn((double)y, cy), dx = __dsub_rn((double)x, cx);
+            if (__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)) <= r2) {
+                s0 += v;
+                sx += (unsigned long long)x * v;
+                sy += (unsigned long long)y * v;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            sx += __shfl_xor_sync(0xffffffffu, sx, o);
+            sy += __shfl_xor_sync(0xffffffffu, sy, o);
+        }
+        if (s0 > 0) {
+            cx = __ddiv_rn((double)sx, (double)s0);
+            cy = __ddiv_rn((double)sy, (double)s0);
+        }
+    }
+    if (lane == 0) out[p] = make_float2((float)cx, (float)cy);
+}
+
 }  // namespace
 
 cudaError_t launch_find_centres(const void* frames, int dtype, int64_t n, int H, int W, double cx0, double cy0,
@@ -54,6 +98,14 @@ cudaError_t launch_find_centres(const void* frames, int dtype, int64_t n, int H,
     if (n <= 0) return cudaSuccess;
     const int threads = 128;
     const int64_t grid = (n + threads - 1) / threads;
+    // exact in any order while pixels x value x coordinate stays below 2^53
+    const double side = 2.0 * radius + 1.0;
+    const double pixels = (side < W ? side : W) * (side < H ? side : H);
+    if (dtype == TM_DTYPE_U16 && pixels * 65535.0 * (W > H ? W : H) < 9.0e15 && pixels < 2.0e9) {
+        find_centres_u16_kernel<<<(unsigned)((n + 3) / 4), threads, 0, st>>>((const uint16_t*)frames, n, H, W, cx0, cy0,
+                                                                            radius, iterations, out);
+        return cudaGetLastError();
+    }
     if (dtype == TM_DTYPE_U16)
         find_centres_kernel<uint16_t><<<(unsigned)grid, threads, 0, st>>>((const uint16_t*)frames, n, H, W, cx0, cy0,
                                                                           radius, iterations, out);

@@ -1309,10 +1309,22 @@ int tm_preprocess(tm_ctx* ctx, const tm_preprocess_params* pp, const void* frame
     int rc = workspace(ctx, st, "pre_weights", w.size() * sizeof(float), (void**)&dw);
     const size_t img = (size_t)n * H * W * sizeof(float);
     float *t1 = nullptr, *t2 = nullptr;
-    if (!rc) rc = workspace(ctx, st, "pre_t1", img, (void**)&t1);
-    if (!rc && dog) rc = workspace(ctx, st, "pre_t2", img, (void**)&t2);
+    // one pass over memory where the rolling rows fit (the output may be the input: not then, as a
+    // band reads rows that another one writes)
+    const char *ib = (const char*)frames_dev, *ob = (const char*)out_dev;
+    const size_t in_bytes = (size_t)n * H * W * (dtype == TM_DTYPE_U16 ? 2 : 4);
+    const bool apart = ob + img <= ib || ib + in_bytes <= ob;
+    const bool stream_pass = apart && tmgb::gauss_stream_supported(W, r_min, r_max, r_blur, dog, blur);
+    if (!rc && !stream_pass) rc = workspace(ctx, st, "pre_t1", img, (void**)&t1);
+    if (!rc && !stream_pass && dog) rc = workspace(ctx, st, "pre_t2", img, (void**)&t2);
     if (rc) return rc;
     TM_CUDA(cudaMemcpyAsync(dw, w.data(), w.size() * sizeof(float), cudaMemcpyHostToDevice, st), "tm_preprocess: weights");
+    if (stream_pass) {
+        TM_CUDA(tmgb::launch_gauss_stream(frames_dev, dtype, n, H, W, dw + o_min, r_min, dw + o_max, r_max, dw + o_blur,
+                                          r_blur, dog, blur, out_dev, ctx->num_sms, st),
+                "tm_preprocess: stream");
+        return TM_OK;
+    }
     const int64_t rows = n * (int64_t)H;
     if (dog) {
         TM_CUDA(tmgb::launch_gauss_rows(frames_dev, dtype, rows, W, dw + o_min, r_min, dw + o_max, r_max, t1, t2, st),

@@ -147,3 +147,24 @@ def test_index_after_background_removal(ctx):
         ok += int(k == ref["template"][p, 0] or abs(ref["q_best"][p, k] - qb) <= 1e-4 * abs(qb))
     assert ok >= 0.98 * frames.shape[0], ok
     ctx.unload_library(lid)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,H,W,dog,blur", [
+    (1, 256, 256, (1.0, 4.0), 1.0), (700, 40, 31, (1.0, 4.0), 1.0), (5, 5, 8, (1.0, 4.0), 2.0),
+    (3, 250, 243, (0.3, 0.6), 0.5), (2, 33, 65, (2.0, 5.3), 0.0), (9, 17, 300, None, 3.0), (400, 64, 9, None, 0.2),
+    (4, 100, 400, (1.5, 2.5), 4.0)])
+def test_one_pass_equals_the_separate_passes(n, H, W, dog, blur):
+    """The one-pass kernel gives the bits of the row and column kernels, which still serve a result
+    written over its input."""
+    import torch
+    ctx = tmgb.Context(0)
+    rng = np.random.default_rng(n * 1000 + H)
+    frames = torch.from_numpy(rng.poisson(3.0, size=(n, H, W)).astype(np.float32)).cuda()
+    apart = ctx.preprocess(frames, dog=dog, blur=blur)
+    over = frames.clone()
+    ctx.preprocess(over, dog=dog, blur=blur, out=over)
+    assert torch.equal(apart, over)
+    u16 = ctx.preprocess(torch.from_numpy(frames.cpu().numpy().astype(np.uint16)).cuda(), dog=dog, blur=blur)
+    assert torch.equal(apart, u16)
+    ctx.close()
