@@ -22,9 +22,14 @@
 //
 // window_kernel: one CTA per pattern; piece maxima of the library's rows, then the W columns.
 // bound_templates_kernel: B, one warp per template (once per library).
-// bound_kernel: the contraction.  D[128 templates x 240 columns] per unit = 240 / nw patterns;
+// bound_kernel: the contraction (32768 patterns against the 13986-template HCP library, six windows:
+//   2.0 ms; 2.55 ms before the issuing threads were freed of divisions and descriptor arithmetic, and
+//   2.3 ms without the clusters' multicast; its loads alone, its MMAs alone and its epilogue alone take
+//   within a fifth of each other).  D[128 templates x 240 columns] per unit = 240 / nw patterns;
 //   a persistent CTA keeps its 128 templates' B (kd <= 512: at most 128 KB) in shared memory and
-//   streams W through a ring; two accumulators in TMEM (columns 0 and 256), so the epilogue of one
+//   streams W through a ring.  Two CTAs form a cluster over two neighbouring template tiles and the
+//   same columns: each loads half of every W chunk into both (multicast), so L2 gives each byte once
+//   for both.  Two accumulators in TMEM (columns 0 and 256), so the epilogue of one
 //   unit runs beside the MMAs of the next.  Units are ordered in blocks of kSuper column tiles
 //   (W of one block: 15 MB, kept in L2 while every template tile passes over it).  Warps: 0 TMA
 //   producer, 1 MMA issuer, 2 TMEM allocation, 4-11 epilogue (TMEM lane quadrant x column half):
@@ -51,6 +56,7 @@ constexpr int kAChunk = kM * kChunkK * 2;  // 16 KB
 constexpr int kBChunk = kN * kChunkK * 2;  // 30 KB
 constexpr int kMaxStages = 5;
 constexpr int kAccStride = 256;            // TMEM columns between the two accumulators
+constexpr int kPair = 2;                   // CTAs of a cluster: neighbouring template tiles, the same columns
 constexpr int kSuper = 64;                 // column tiles per block of units
 constexpr int kEpi0 = 4, kEpiThreads = 256;
 constexpr int kBoundThreads = kEpi0 * 32 + kEpiThreads;
@@ -213,11 +219,12 @@ bound_templates_kernel(const int4* __restrict__ meta, const int4* __restrict__ o
 }
 
 struct Units {                                             // the order of a CTA's units
-    int mt, nt;                                            // template tiles, column tiles
+    int mt, nt;                                            // pairs of template tiles, column tiles
+    int cluster, clusters;                                 // this CTA's cluster of how many
     __device__ __forceinline__ int super(int s) const { return min(kSuper, nt - s * kSuper); }
 };
 
-// Calls f(template tile, column tile, first unit of a template tile, last unit of it) for the CTA's
+// Calls f(pair of template tiles, column tile, first unit of a pair, last unit of it) for the cluster's
 // units; stops when f returns false.
 template <typename F>
 __device__ __forceinline__ void for_units(const Units& g, F f) {
@@ -226,26 +233,31 @@ __device__ __forceinline__ void for_units(const Units& g, F f) {
     for (int s = 0; s < supers; ++s) {
         const int sb = g.super(s);
         const int64_t total = (int64_t)g.mt * sb;
-        const int64_t lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
+        const int64_t lo = total * g.cluster / g.clusters, hi = total * (g.cluster + 1) / g.clusters;
         // whether the units of the next block (if the CTA has any) go on with the same template tile
         int next_mt = -1;
         for (int s2 = s + 1; s2 < supers && next_mt < 0; ++s2) {
             const int sb2 = g.super(s2);
             const int64_t t2 = (int64_t)g.mt * sb2;
-            const int64_t l2 = t2 * blockIdx.x / gridDim.x, h2 = t2 * (blockIdx.x + 1) / gridDim.x;
+            const int64_t l2 = t2 * g.cluster / g.clusters, h2 = t2 * (g.cluster + 1) / g.clusters;
             if (l2 < h2) next_mt = (int)(l2 / sb2);
         }
-        for (int64_t u = lo; u < hi; ++u) {
-            const int m = (int)(u / sb), c = s * kSuper + (int)(u - (int64_t)m * sb);
-            const int after = u + 1 < hi ? (int)((u + 1) / sb) : next_mt;
-            if (!f(m, c, m != prev, after != m)) return;
+        // (counted on, not divided: a 64-bit division a unit in every role had been a quarter of the time)
+        const int count = (int)(hi - lo);
+        int m = (int)(lo / sb), c = (int)(lo - (int64_t)m * sb);
+        for (int i = 0; i < count; ++i) {
+            const bool row_ends = c + 1 == sb;
+            const int after = i + 1 < count ? (row_ends ? m + 1 : m) : next_mt;
+            if (!f(m, s * kSuper + c, m != prev, after != m)) return;
             prev = m;
+            c = row_ends ? 0 : c + 1;
+            m += row_ends;
         }
     }
 }
 
 template <int NW>
-__global__ void __launch_bounds__(kBoundThreads, 1)
+__global__ void __cluster_dims__(kPair, 1, 1) __launch_bounds__(kBoundThreads, 1)
 bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap, const BoundCall c) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -253,7 +265,7 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
     const int stages = c.stages;
     uint8_t* s_a = base;                                    // chunks x 16 KB
     uint8_t* s_b = s_a + chunks * kAChunk;                  // stages x 30 KB
-    __shared__ uint64_t bar[2 * kMaxStages + 6];            // full[S], empty[S], a_full, a_empty, acc_full[2], acc_empty[2]
+    __shared__ uint64_t bar[2 * kMaxStages + 7];            // full[S], empty[S], a_full, a_empty, acc_full[2], acc_empty[2], done
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     __shared__ int s_stop[2];
@@ -262,21 +274,26 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
     const uint32_t full0 = smem_u32(&bar[0]), empty0 = smem_u32(&bar[kMaxStages]);
     const uint32_t a_full = smem_u32(&bar[2 * kMaxStages]), a_empty = smem_u32(&bar[2 * kMaxStages + 1]);
     const uint32_t accf0 = smem_u32(&bar[2 * kMaxStages + 2]), acce0 = smem_u32(&bar[2 * kMaxStages + 4]);
+    const uint32_t done = smem_u32(&bar[2 * kMaxStages + 6]);   // MMAs finished, when stopping
     constexpr int kPat = kN / NW;                           // patterns per unit
     Units g;
-    g.mt = (c.K + kM - 1) / kM;
+    const int rank = blockIdx.x % kPair;
+    g.mt = (c.K + kM * kPair - 1) / (kM * kPair);
+    g.cluster = blockIdx.x / kPair;
+    g.clusters = gridDim.x / kPair;
     g.nt = (int)((c.n + kPat - 1) / kPat);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kMaxStages; ++i) {
             mbar_init(full0 + 8 * i, 1);
-            mbar_init(empty0 + 8 * i, 1);
+            mbar_init(empty0 + 8 * i, kPair);               // both CTAs' MMAs have read the slot
         }
         mbar_init(a_full, 1);
         mbar_init(a_empty, 1);
+        mbar_init(done, 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(accf0 + 8 * i, 1);
-            mbar_init(acce0 + 8 * i, kEpiThreads);
+            mbar_init(acce0 + 8 * i, kEpiThreads / 32);
         }
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -290,6 +307,7 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync();                                         // (the peer's barriers are initialised as well)
     tc_fence_after();
     const uint32_t tmem = s_tmem;
 
@@ -297,27 +315,32 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
         // ================================================================ TMA producer
         if (lane == 0) {
             uint32_t q = 0, na = 0;                         // ring chunks and template tiles loaded
+            uint32_t slot = 0, phase = 0;                   // of the next chunk (counted on, not divided)
             for_units(g, [&](int m, int ct, bool first, bool) {
                 if (first) {
                     if (!mbar_wait(a_empty, (na & 1u) ^ 1u, abort_flag)) { *abort_flag = 1; return false; }
                     mbar_expect_tx(a_full, (uint32_t)(chunks * kAChunk));
                     for (int ch = 0; ch < chunks; ++ch)
-                        tma_load_2d(smem_u32(s_a + ch * kAChunk), &amap, ch * kChunkK, m * kM, a_full);
+                        tma_load_2d(smem_u32(s_a + ch * kAChunk), &amap, ch * kChunkK, (m * kPair + rank) * kM, a_full);
                     ++na;
                 }
                 for (int ch = 0; ch < chunks; ++ch, ++q) {
-                    const uint32_t slot = q % stages, use = q / stages;
-                    if (!mbar_wait(empty0 + 8 * slot, (use & 1u) ^ 1u, abort_flag)) { *abort_flag = 1; return false; }
+                    if (!mbar_wait(empty0 + 8 * slot, phase ^ 1u, abort_flag)) { *abort_flag = 1; return false; }
                     mbar_expect_tx(full0 + 8 * slot, kBChunk);
-                    tma_load_2d(smem_u32(s_b + slot * kBChunk), &bmap, ch * kChunkK, ct * kN, full0 + 8 * slot);
+                    // this CTA's half of the chunk's rows, into both
+                    tma_load_2d_multicast(smem_u32(s_b + slot * kBChunk + rank * (kBChunk / kPair)), &bmap, ch * kChunkK,
+                                          ct * kN + rank * (kN / kPair), full0 + 8 * slot, (1u << kPair) - 1);
+                    if (++slot == (uint32_t)stages) { slot = 0; phase ^= 1u; }
                 }
                 return true;
             });
-            // the copies issued last must land before the CTA exits (they complete on their own)
+            // the copies issued last must land, and both CTAs' MMAs have reported their slots read, before
+            // the CTA exits (they complete on their own)
             volatile int never = 0;
             for (uint32_t i = 0; i < (uint32_t)stages && i < q; ++i) {
-                const uint32_t qq = q - 1 - i;
-                mbar_wait(full0 + 8 * (qq % stages), (qq / stages) & 1u, &never);
+                const uint32_t qq = q - 1 - i, slot = qq % stages, par = (qq / stages) & 1u;
+                mbar_wait(full0 + 8 * slot, par, &never);
+                mbar_wait(empty0 + 8 * slot, par, abort_flag);
             }
             if (na) mbar_wait(a_full, (na - 1) & 1u, &never);
         }
@@ -325,10 +348,9 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
         // ================================================================ MMA issuer
         if (lane == 0) {
             const uint32_t idesc = idesc_f16(kM, kN);
-            const uint32_t a0 = smem_u32(s_a), b0 = smem_u32(s_b);
-            uint32_t q = 0, na = 0, tt = 0;
+            const uint64_t a_desc = sdesc_kmajor(smem_u32(s_a)), b_desc = sdesc_kmajor(smem_u32(s_b));
+            uint32_t na = 0, tt = 0, slot = 0, phase = 0;
             bool stop = false, issued = false;
-            uint32_t last_bar = 0, last_par = 0;
             for_units(g, [&](int, int, bool first, bool last) {
                 if (first) {
                     if (!mbar_wait(a_full, na & 1u, abort_flag)) { stop = true; return false; }
@@ -338,18 +360,20 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
                 if (!mbar_wait(acce0 + 8 * buf, ((tt >> 1) & 1u) ^ 1u, abort_flag)) { stop = true; return false; }
                 tc_fence_after();
                 const uint32_t d = tmem + buf * kAccStride;
-                for (int ch = 0; ch < chunks; ++ch, ++q) {
-                    const uint32_t slot = q % stages, use = q / stages;
-                    if (!mbar_wait(full0 + 8 * slot, use & 1u, abort_flag)) { stop = true; return false; }
+                for (int ch = 0; ch < chunks; ++ch) {
+                    if (!mbar_wait(full0 + 8 * slot, phase, abort_flag)) { stop = true; return false; }
                     tc_fence_after();
-                    const int ks_n = min(kChunkK / 16, steps - ch * (kChunkK / 16));
-                    for (int ks = 0; ks < ks_n; ++ks)
-                        mma_f16(d, sdesc_kmajor(a0 + ch * kAChunk + ks * 32), sdesc_kmajor(b0 + slot * kBChunk + ks * 32),
-                                idesc, (ch | ks) ? 1u : 0u);
-                    mma_commit(empty0 + 8 * slot);
-                    last_bar = empty0 + 8 * slot;
-                    last_par = use & 1u;
+                    // (descriptors counted on from the chunk's: an MMA takes 127 clocks, and building
+                    // both from scratch for each had taken the issuing thread longer than that)
+                    const uint64_t da = a_desc + (uint64_t)(ch * (kAChunk >> 4));
+                    const uint64_t db = b_desc + (uint64_t)(slot * (kBChunk >> 4));
+                    const int ks_n = steps - ch * (kChunkK / 16);
+#pragma unroll
+                    for (int ks = 0; ks < kChunkK / 16; ++ks)
+                        if (ks < ks_n) mma_f16(d, da + 2 * ks, db + 2 * ks, idesc, (ch | ks) ? 1u : 0u);
+                    mma_commit_multicast(empty0 + 8 * slot, (1u << kPair) - 1);
                     issued = true;
+                    if (++slot == (uint32_t)stages) { slot = 0; phase ^= 1u; }
                 }
                 if (last) mma_commit(a_empty);
                 mma_commit(accf0 + 8 * buf);
@@ -360,7 +384,8 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
                 *abort_flag = 1;
                 if (issued) {                               // let the MMAs already issued finish
                     volatile int never = 0;
-                    mbar_wait(last_bar, last_par, &never);
+                    mma_commit(done);
+                    mbar_wait(done, 0, &never);
                 }
             }
         }
@@ -386,8 +411,9 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
             uint32_t r[kHalf];
             tmem_ld120(tb + buf * kAccStride, r);
             tc_fence_before();
-            mbar_arrive(acce0 + 8 * buf);                   // the accumulator is in registers
-            const int k = m * kM + quad * 32 + lane, word = m * (kM / 32) + quad;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acce0 + 8 * buf);    // the accumulator is in registers
+            const int k = (m * kPair + rank) * kM + quad * 32 + lane, word = (m * kPair + rank) * (kM / 32) + quad;
             const int64_t p0 = (int64_t)ct * kPat + half * kMine;
             uint32_t wm = 0;                                // lane i: the word's maximum for pattern i
 #pragma unroll
@@ -410,6 +436,7 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    cluster_sync();                                         // the peer's copies and arrivals into this CTA are done
     if (*abort_flag && threadIdx.x == 0) atomicOr(c.error, 8u);
     if (warp == 2) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
@@ -465,7 +492,7 @@ cudaError_t launch_bound_windows(const float* polar, const float* pnorm, int64_t
     return cudaGetLastError();
 }
 
-int bound_box_rows(bool templates) { return templates ? kM : kN; }
+int bound_box_rows(bool templates) { return templates ? kM : kN / kPair; }
 
 cudaError_t launch_bound(const void* amap, const void* bmap, const BoundCall& call, int nw, int num_sms,
                          cudaStream_t st) {
@@ -478,8 +505,13 @@ cudaError_t launch_bound(const void* amap, const void* bmap, const BoundCall& ca
     const cudaError_t e = kernel_occupancy(fn, kBoundThreads, smem, nullptr);
     if (e != cudaSuccess) return e;
     const int pat = kN / nw;
-    const int64_t units = (int64_t)((c.K + kM - 1) / kM) * ((c.n + pat - 1) / pat);
-    const int grid = (int)std::min<int64_t>(num_sms, units);
+    const int64_t units = (int64_t)((c.K + kM * kPair - 1) / (kM * kPair)) * ((c.n + pat - 1) / pat);
+    // no more clusters than run at once: the units are split evenly between them
+    int clusters = 0;
+    const cudaError_t ec = cluster_occupancy(fn, kBoundThreads, smem, kPair, &clusters);
+    if (ec != cudaSuccess) return ec;
+    clusters = std::min(clusters, num_sms / kPair);
+    const int grid = kPair * (int)std::max<int64_t>(1, std::min<int64_t>(clusters, units));
     if (nw == 12)
         bound_kernel<12><<<grid, kBoundThreads, smem, st>>>(*(const CUtensorMap*)amap, *(const CUtensorMap*)bmap, c);
     else

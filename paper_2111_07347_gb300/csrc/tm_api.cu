@@ -161,6 +161,33 @@ cudaError_t kernel_occupancy(const void* fn, int threads, size_t smem, int* per_
     return cudaSuccess;
 }
 
+cudaError_t cluster_occupancy(const void* fn, int threads, size_t smem, int size, int* clusters) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(g_launch_mu);
+    const auto key = std::make_tuple(fn, dev, -threads, smem);   // (negative: clusters, not blocks)
+    auto it = g_occupancy.find(key);
+    if (it == g_occupancy.end()) {
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = size;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(size);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
+        if (e != cudaSuccess) return e;
+        it = g_occupancy.emplace(key, n).first;
+    }
+    *clusters = it->second;
+    return cudaSuccess;
+}
+
 namespace {
 thread_local int t_sm_cap = 0;      // persistent grids of this thread's calls use at most this many SMs
 }
@@ -673,23 +700,24 @@ uint16_t f32_to_bf16(float f) {
     return (uint16_t)(u >> 16);
 }
 
-// Inverse-DFT basis for the radix-2 split (rows: shift s < n/2; columns: even-m then odd-m
-// (re, im) pairs) and the twiddle table, built in FP64 and cached per n_theta.
+// Inverse-DFT basis for the radix-2 splits (rows: shifts s <= n/4 of the even, then of the odd
+// frequencies; columns: the cosines, then the sines of the part's slots) and the twiddle table, built in FP64 and cached per n_theta.
 int spectral_tables(tm_ctx* ctx, int n_theta, SpectralTables* out) {
     auto it = ctx->spectral.find(n_theta);
     if (it == ctx->spectral.end()) {
         const int R = tmgb::dense_basis_rows(), C = tmgb::dense_basis_cols(), half = C / 2;
         const int H = n_theta / 2;
         std::vector<uint16_t> basis((size_t)R * C, 0);
-        for (int s = 0; s < R && s < H; ++s) {
+        for (int row = 0; row < R; ++row) {
+            // even, then odd frequencies; rows past the last shift repeat it
+            const int part = row / (R / 2), s = std::min(row % (R / 2), H / 2);
             for (int kk = 0; kk < C; ++kk) {
-                const int part = kk / half, j = (kk % half) / 2, comp = kk % 2;
-                const int m = 2 * j + part;
+                const int m = 2 * (kk % half) + part;
                 if (m > H) continue;
                 const double w = (m == 0 || m == H) ? 1.0 : 2.0;
                 const double ang = 2.0 * kPi * (double)m * (double)s / n_theta;
-                const double v = (w / n_theta) * (comp == 0 ? cos(ang) : -sin(ang));
-                basis[(size_t)s * C + kk] = f32_to_bf16((float)v);
+                const double v = (w / n_theta) * (kk < half ? cos(ang) : -sin(ang));
+                basis[(size_t)row * C + kk] = f32_to_bf16((float)v);
             }
         }
         std::vector<float2> tw(n_theta);
@@ -925,16 +953,23 @@ int bound_tensor_map(tm_ctx* ctx, void* base, int64_t rows, int pitch, int box_r
     return TM_OK;
 }
 
-// Tensor map of G [192][nb][2][K_pad] BF16 for stage B: 4-D (k, c, p, j), boxes of
-// 64 templates x 2 x 1 pattern x 32 slots, 128-byte swizzle, zero fill past K.
-int g_tensor_map(tm_ctx* ctx, void* g, int K, int K_pad, int64_t nb, CUtensorMap* out) {
+// Frequencies of the even and odd slots: m = 2 j <= n / 2 and m = 2 j + 1 <= n / 2.
+inline int even_slots(int n_theta) { return n_theta / 4 + 1; }
+inline int odd_slots(int n_theta) { return (n_theta / 2 + 1) / 2; }
+
+// Tensor map of `slots` slots from slot `first` of G [192][nb][2][K_pad] BF16 for stage B: 4-D
+// (k, c, p, j), boxes of 64 templates x 1 x 1 pattern x box_rows slots, 128-byte swizzle, zero fill
+// past K and past the slots.
+int g_tensor_map(tm_ctx* ctx, void* g, int K, int K_pad, int64_t nb, int first, int slots, int box_rows,
+                 CUtensorMap* out) {
     const int rc = tensor_map_encoder(ctx);
     if (rc) return rc;
-    const cuuint64_t dims[4] = {(cuuint64_t)K, 2, (cuuint64_t)nb, (cuuint64_t)tmgb::dense_slots()};
+    const cuuint64_t dims[4] = {(cuuint64_t)K, 2, (cuuint64_t)nb, (cuuint64_t)slots};
     const cuuint64_t strides[3] = {(cuuint64_t)K_pad * 2, (cuuint64_t)K_pad * 4, (cuuint64_t)nb * K_pad * 4};
-    const cuuint32_t box[4] = {64, 2, 1, 32};
+    const cuuint32_t box[4] = {64, 1, 1, (cuuint32_t)box_rows};
     const cuuint32_t es[4] = {1, 1, 1, 1};
-    const CUresult r = ctx->encode_tiled(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, g, dims, strides, box, es,
+    void* base = (char*)g + (size_t)first * nb * K_pad * 4;
+    const CUresult r = ctx->encode_tiled(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, es,
                                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(TM_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
@@ -983,11 +1018,17 @@ int stage_a(tm_ctx* ctx, cudaStream_t st, const Library* L, const TensorBuffers&
     cublasStatus_t s = CUBLAS_STATUS_SUCCESS;
     const float one = 1.0f, zero = 0.0f;
     const int R2 = 2 * L->R;
-    s = cublasGemmStridedBatchedEx(ctx->cublas, CUBLAS_OP_N, CUBLAS_OP_N, L->K_pad, (int)(2 * nb), R2, &one,
-                                   L->d_that, CUDA_R_16BF, L->K_pad, (long long)R2 * L->K_pad, tb.phat, CUDA_R_16BF,
-                                   R2, (long long)nb * 2 * R2, &zero, tb.g, CUDA_R_16BF, L->K_pad,
-                                   (long long)2 * nb * L->K_pad, tmgb::dense_slots(), CUBLAS_COMPUTE_32F,
-                                   CUBLAS_GEMM_DEFAULT);
+    // the slots that hold a frequency (stage B reads no others)
+    const int slots = tmgb::dense_slots(), first[2] = {0, slots / 2}, count[2] = {even_slots(L->n_theta), odd_slots(L->n_theta)};
+    for (int i = 0; i < 2 && s == CUBLAS_STATUS_SUCCESS; ++i) {
+        const size_t j = (size_t)first[i];
+        s = cublasGemmStridedBatchedEx(ctx->cublas, CUBLAS_OP_N, CUBLAS_OP_N, L->K_pad, (int)(2 * nb), R2, &one,
+                                       (const uint16_t*)L->d_that + j * R2 * L->K_pad, CUDA_R_16BF, L->K_pad,
+                                       (long long)R2 * L->K_pad, (const uint16_t*)tb.phat + j * nb * 2 * R2, CUDA_R_16BF,
+                                       R2, (long long)nb * 2 * R2, &zero, (uint16_t*)tb.g + j * 2 * nb * L->K_pad,
+                                       CUDA_R_16BF, L->K_pad, (long long)2 * nb * L->K_pad, count[i], CUBLAS_COMPUTE_32F,
+                                       CUBLAS_GEMM_DEFAULT);
+    }
     if (s != CUBLAS_STATUS_SUCCESS) return fail(TM_ERR_CUDA, "stage A GEMM failed (cuBLAS status %d)", (int)s);
     return TM_OK;
 }
@@ -1021,10 +1062,15 @@ int prescore_rows(tm_ctx* ctx, cudaStream_t st, Library* const* libs, int n_libs
                 const int rc = stage_a(ctx, st, L, tb, nb);
                 if (rc) return rc;
             }
-            CUtensorMap map;
-            const int rc = g_tensor_map(ctx, tb.g, (int)L->K, L->K_pad, nb, &map);
+            CUtensorMap emap, omap;
+            const int ne = even_slots(n_theta), box_rows = (ne + 15) & ~15;   // (as many odd slots, or one less)
+            int rc = g_tensor_map(ctx, tb.g, (int)L->K, L->K_pad, nb, 0, ne, box_rows, &emap);
+            if (!rc)
+                rc = g_tensor_map(ctx, tb.g, (int)L->K, L->K_pad, nb, tmgb::dense_slots() / 2, odd_slots(n_theta), box_rows,
+                                  &omap);
             if (rc) return rc;
             tmgb::DenseCall dc{};
+            dc.box_rows = box_rows;
             dc.n = nb;
             dc.p0 = b0;
             dc.n_theta = n_theta;
@@ -1037,7 +1083,7 @@ int prescore_rows(tm_ctx* ctx, cudaStream_t st, Library* const* libs, int n_libs
             dc.stall = stall;
             {
                 StageTimer tmr(ctx, TM_STAGE_DENSE, st);
-                TM_CUDA(tmgb::launch_dense(&map, dc, tmgb::device_sms(), st), "tensor path: stage B");
+                TM_CUDA(tmgb::launch_dense(&emap, &omap, dc, tmgb::device_sms(), st), "tensor path: stage B");
             }
             *launches += 2;              // this library's kernels (the GEMMs are cuBLAS's)
         }

@@ -77,6 +77,9 @@ struct RadialLib {
 // returns its resident blocks per SM for `threads` threads (per_sm may be null).  Cached, so
 // repeated launches make no driver queries.
 cudaError_t kernel_occupancy(const void* fn, int threads, size_t smem, int* per_sm);
+// Clusters of `size` blocks that are resident at once on the device (cached; after kernel_occupancy
+// has raised the limit).
+cudaError_t cluster_occupancy(const void* fn, int threads, size_t smem, int size, int* clusters);
 // Number of SMs of the current device (cached), or the calling thread's cap when one is set.
 int device_sms();
 // Caps the persistent grids of this thread's later calls at `cap` SMs (0 = no cap), so that work
@@ -285,7 +288,8 @@ struct DenseCall {
     int64_t p0;                // first pattern of the batch in the call's rows (pre, mask)
     int n_theta;
     int K;                     // templates of the library
-    const void* basis;         // [192][384] bf16, K-major (dense_basis_rows x dense_basis_cols)
+    const void* basis;         // [2][96][192] bf16, K-major (dense_basis_rows x dense_basis_cols)
+    int box_rows;              // slots of a part, a multiple of 16 (the tensor maps' boxes)
     const uint32_t* mask;      // [rows][words] templates to score (pre-filter) or null (all)
     int words;
     float* pre;                // [rows][K] out: pre-score, -NaN where masked out
@@ -298,8 +302,9 @@ int dense_basis_rows();
 int dense_basis_cols();
 int dense_slots();
 size_t dense_smem_bytes();
-// tmap: the CUtensorMap of G for this batch (4-D: k, c, p, j; box 64 x 2 x 1 x 32; 128-byte swizzle).
-cudaError_t launch_dense(const void* tmap, const DenseCall& c, int num_sms, cudaStream_t st);
+// emap, omap: the CUtensorMaps of G's even and odd slots for this batch (4-D: k, c, p, j; box
+// 64 x 1 x 1 x box_rows; 128-byte swizzle; slots past n_theta / 2 out of bounds, read as zero).
+cudaError_t launch_dense(const void* emap, const void* omap, const DenseCall& c, int num_sms, cudaStream_t st);
 // dftc [192][2][nb][n_r] FP32 (the DFT GEMM's output for every polar row) -> P^ of one library
 // [192][nb][2][2 R] BF16, divided by |P|.
 cudaError_t launch_pack(const float* dftc, const float* pnorm, int64_t nb, int n_r, const int32_t* radii, int n_rad,

@@ -44,7 +44,7 @@ __device__ __forceinline__ bool mbar_try_addr(uint32_t addr, uint32_t parity) {
 }
 
 // Bounded wait; false on timeout or when another role has aborted.
-static __device__ bool mbar_wait(uint32_t addr, uint32_t parity, volatile int* abort_flag) {
+static __device__ __noinline__ bool mbar_wait_slow(uint32_t addr, uint32_t parity, volatile int* abort_flag) {
     uint64_t t0 = 0;
     for (uint32_t it = 0;; ++it) {
         if (mbar_try_addr(addr, parity)) return true;
@@ -55,6 +55,9 @@ static __device__ bool mbar_wait(uint32_t addr, uint32_t parity, volatile int* a
             else if (t - t0 > kTimeoutNs) return false;
         }
     }
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, volatile int* abort_flag) {
+    return mbar_try_addr(addr, parity) || mbar_wait_slow(addr, parity, abort_flag);
 }
 
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -116,6 +119,30 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         "[%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
         "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(mbar)
         : "memory");
+}
+
+// The same copy into the shared memory of every CTA of `mask` in the cluster, at the same offset,
+// completing on the mbarrier at the same offset in each.
+__device__ __forceinline__ void tma_load_2d_multicast(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t mbar,
+                                                      uint16_t mask) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster "
+        "[%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+        "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(mbar), "h"(mask)
+        : "memory");
+}
+
+// Arrives, once this thread's earlier MMAs are done, on the mbarrier at the same offset in every CTA
+// of `mask` in the cluster.
+__device__ __forceinline__ void mma_commit_multicast(uint32_t mbar, uint16_t mask) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(mbar),
+        "h"(mask)
+        : "memory");
+}
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
 }  // namespace tmgb
