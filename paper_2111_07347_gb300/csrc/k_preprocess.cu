@@ -526,8 +526,18 @@ cudaError_t launch_stream(const T* in, int64_t n, int H, int W, const float* w1,
     const cudaError_t e = kernel_occupancy((const void*)gauss_stream_kernel<T, PITCH>, kStreamThreads, smem, &per_sm);
     if (e != cudaSuccess) return e;
     const int64_t slots = (int64_t)num_sms * std::max(1, per_sm);
-    // one band a frame while the frames fill the GPU; else bands of at least 16 rows
-    int bands = (int)std::min<int64_t>((slots + n - 1) / n, (H + 15) / 16);
+    // one band a frame while the frames fill the GPU; else the number of bands (of at least 16 rows)
+    // with the fewest row steps, counting the reach that each band repeats at its ends and the waves
+    const int reach = 2 * (s.R + s.rb);
+    int bands = 1;
+    int64_t least = INT64_MAX;
+    for (int b = 1; b <= std::max(1, H / 16) && (b == 1 || n < slots); ++b) {
+        const int64_t cost = ((n * b + slots - 1) / slots) * ((H + b - 1) / b + kB - 1 + reach);
+        if (cost < least) {
+            least = cost;
+            bands = b;
+        }
+    }
     const int band_rows = ((H + bands - 1) / bands + kB - 1) / kB * kB;
     bands = (H + band_rows - 1) / band_rows;
     const int grid = (int)std::min<int64_t>(n * bands, slots);
