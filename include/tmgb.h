@@ -296,7 +296,7 @@ int tm_index_patterns(tm_ctx* ctx, const tm_index_params* params, const void* fr
 
 /* The whole path (as tm_index_patterns) for frames and results in HOST memory.  The paper's
  * GPU implementation moves each image to the device before indexing it (Section 2.2); here
- * the batch is cut into chunks of `chunk` patterns (0: 4096) that alternate between two
+ * the batch is cut into chunks of `chunk` patterns (0: an eighth of the batch, 512 to 4096) that alternate between two
  * streams owned by the context, so the host->device copy of one chunk overlaps the kernels
  * of the previous one, and each chunk's hits are copied back as soon as they are ready.
  * frames_host [n][H][W] (dtype), centres_host [n][2] float or NULL, out_host

@@ -1180,7 +1180,10 @@ int tm_index_patterns_host(tm_ctx* ctx, const tm_index_params* params, const voi
     if (stats) memset(stats, 0, sizeof *stats);
     if (n == 0) return TM_OK;
     if (!frames_host || !out_host) return fail(TM_ERR_INVALID_ARG, "tm_index_patterns_host: NULL buffer");
-    if (chunk == 0) chunk = 4096;
+    // default: eight chunks, so that little of the first copy and of the last chunk's kernels is left
+    // uncovered, of 512 to 4096 patterns (8192 frames of 256 x 256: 5.58 ms, chunks of 4096
+    // 6.43 ms; 2048 frames 1.59 and 2.01 ms)
+    if (chunk == 0) chunk = std::min<int64_t>(4096, std::max<int64_t>(512, (n + 7) / 8));
     if (chunk > n) chunk = n;
     std::lock_guard<std::mutex> hl(ctx->host_mu);
     DeviceGuard g(ctx->device);
