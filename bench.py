@@ -557,10 +557,11 @@ class Timer:
 
 
 def sparse_roofline(prof, counters, prof_steps, macs_step, clk, sm, patterns_step):
-    """Shared-memory roofline of sparse_kernel: one 4-byte operand per FP32 multiply-add.  frac is
-    the executed work (the multiply-adds the kernel ran, counted while profiling) over the peak;
-    the algorithmic fraction counts every template the definition scores, including those the
-    exact bound pruning skips."""
+    """Shared-memory roofline of the FP32 scoring stage (bounds on the tensor cores, then exact scores:
+    window_kernel, bound_kernel, score_kernel; sparse_kernel for the libraries the bounds do not take):
+    one 4-byte operand per FP32 multiply-add.  frac is the executed work (the multiply-adds the
+    scoring kernel ran, counted while profiling) over the stage's time and the peak; the algorithmic
+    fraction counts every template the definition scores, including those the bounds leave out."""
     sp_ms, sp_l = prof.get("sparse", (0.0, 0))
     if not sp_l:
         return None
@@ -572,9 +573,9 @@ def sparse_roofline(prof, counters, prof_steps, macs_step, clk, sm, patterns_ste
     alg = macs_step / lps
     ex_gbs = 4.0 * ex / (per_launch_ms / 1e3) / 1e9
     alg_gbs = 4.0 * alg / (per_launch_ms / 1e3) / 1e9
-    return {"bound": "smem", "kernel": "sparse_kernel", "achieved": ex_gbs, "peak": peak, "unit": "GB/s",
+    return {"bound": "smem", "kernel": "score_kernel (with its bounds)", "achieved": ex_gbs, "peak": peak, "unit": "GB/s",
             "frac": ex_gbs / peak, "traffic": traffic_from_profiles(
-                os.path.join(ROOT, "paper_2111_07347_gb300", "csrc", "k_sparse.cu"), "sparse_kernel",
+                os.path.join(ROOT, "paper_2111_07347_gb300", "csrc", "k_score.cu"), "score_kernel",
                 patterns_step / lps),
             "work": "4 B of shared memory per FP32 multiply-add executed (one polar sample per spot x shift "
                     "of every template the kernel scores)",
