@@ -264,7 +264,7 @@ int tm_prescore(tm_ctx* ctx, int lib_id, const float* polar_dev, const float* no
                 const float* radial_dev, int64_t n, double fraction, float* score_dev, void* stream);
 
 /* Autotune the FP32 sparse kernel for a set of libraries: time its shapes -- block size (128,
- * 256, 512 threads; default 256) x templates seeded per warp for the pruned top-N (4, 8, 16;
+ * 256, 512 threads; by default 256, or 512 where the rows leave an SM two blocks or one) x templates seeded per warp for the pruned top-N (4, 8, 16;
  * default 8: the templates of highest bound are scored first, so that the top-N threshold
  * the others are pruned against starts high) on the first min(n, 2048) frames, then the best
  * of these against its block size with 4 patterns per CTA bounded together (default 1) and

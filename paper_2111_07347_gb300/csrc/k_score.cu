@@ -436,7 +436,7 @@ score_kernel(const ScoreCall c) {
 size_t score_smem(int n_rad, int n_theta, int top_n, int warps, int* layout, int* pitch) {
     if (n_theta < 1 || n_theta > 1024 || top_n < 1 || top_n > TM_MAX_TOPN || n_rad < 1) return 0;
     const int order[2] = {TM_LAYOUT_WF, TM_LAYOUT_WRAP};
-    const size_t limit[2] = {100 * 1024, 227 * 1024};
+    const size_t limit[2] = {113 * 1024, 227 * 1024};
     for (int i = 0; i < 2; ++i) {
         const int pch = sparse_pitch(n_theta, order[i]);
         if (order[i] == TM_LAYOUT_WF && (size_t)n_rad * pch > 65535) continue;   // 16-bit offsets
