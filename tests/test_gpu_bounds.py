@@ -110,3 +110,30 @@ def test_bounds_leave_a_small_budget_to_the_general_path():
         ctx.check()
         ctx.close()
     big.close()
+
+
+@pytest.mark.gpu
+def test_bounds_replay_in_a_graph_and_on_two_streams():
+    """Calls that go through the bounds give the same hits replayed as a CUDA graph, and on two
+    streams whose scratch is their own."""
+    import torch
+    ts = synth.kinematic_library("hcp", step_deg=1.5)
+    scan = synth.render_scan(synth.make_rng(79), ts, 200, 256, 256, n_theta=360)
+    f = torch.from_numpy(scan.frames).cuda()
+    ctx = tmgb.Context(0)
+    lid = ctx.load_library(ts, 128, 360)
+    assert ctx.library_info(lid)["n_templates"] >= 512
+    want = ctx.index(f, lid, top_n=5)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    outs = [torch.zeros_like(want) for _ in streams]
+    for _ in range(4):
+        for st, out in zip(streams, outs):
+            out.zero_()
+        torch.cuda.synchronize()
+        for st, out in zip(streams, outs):
+            ctx.index(f, lid, top_n=5, out=out, stream=st, graph=True)
+        torch.cuda.synchronize()
+        for out in outs:
+            assert torch.equal(out, want)
+    ctx.close()
