@@ -177,8 +177,9 @@ __global__ void __launch_bounds__(kThreads, 1) dense_kernel(const __grid_constan
                     mbar_expect_tx(full, 2 * box);
                     const uint32_t dst = smem_u32(s_ring + slot * kSlotBytes);
                     const CUtensorMap* map = ch < 2 ? &emap : &omap;
-                    tma_load_4d(dst, map, t * kRows, ch & 1, p, 0, full);
-                    tma_load_4d(dst + kBoxBytes, map, t * kRows + 64, ch & 1, p, 0, full);
+                    const int j0 = ch < 2 ? 0 : c.odd_slot;
+                    tma_load_4d(dst, map, t * kRows, ch & 1, p, j0, full);
+                    tma_load_4d(dst + kBoxBytes, map, t * kRows + 64, ch & 1, p, j0, full);
                 }
             }
             // the copies issued last must land before the CTA exits (they complete on their own)

@@ -956,6 +956,10 @@ int bound_tensor_map(tm_ctx* ctx, void* base, int64_t rows, int pitch, int box_r
 // Frequencies of the even and odd slots: m = 2 j <= n / 2 and m = 2 j + 1 <= n / 2.
 inline int even_slots(int n_theta) { return n_theta / 4 + 1; }
 inline int odd_slots(int n_theta) { return (n_theta / 2 + 1) / 2; }
+// Whether a batch's G is small enough that all slots are computed, and read, as one array.
+inline bool whole_slots(const Library* L, int64_t nb) {
+    return (size_t)nb * L->K_pad * tmgb::dense_slots() * 4 < (size_t)256 << 20;
+}
 
 // Tensor map of `slots` slots from slot `first` of G [192][nb][2][K_pad] BF16 for stage B: 4-D
 // (k, c, p, j), boxes of 64 templates x 1 x 1 pattern x box_rows slots, 128-byte swizzle, zero fill
@@ -1018,9 +1022,13 @@ int stage_a(tm_ctx* ctx, cudaStream_t st, const Library* L, const TensorBuffers&
     cublasStatus_t s = CUBLAS_STATUS_SUCCESS;
     const float one = 1.0f, zero = 0.0f;
     const int R2 = 2 * L->R;
-    // the slots that hold a frequency (stage B reads no others)
-    const int slots = tmgb::dense_slots(), first[2] = {0, slots / 2}, count[2] = {even_slots(L->n_theta), odd_slots(L->n_theta)};
-    for (int i = 0; i < 2 && s == CUBLAS_STATUS_SUCCESS; ++i) {
+    // the slots that hold a frequency (stage B reads no others), even and odd ones in a call each; a
+    // small batch takes all slots in one call, as a second launch costs more than the 11 of 192 slots
+    // it would save (at 360 angles they are worth 3 us of HBM writes at 300 MB of G)
+    const int slots = tmgb::dense_slots();
+    const bool whole = whole_slots(L, nb);
+    const int first[2] = {0, slots / 2}, count[2] = {whole ? slots : even_slots(L->n_theta), odd_slots(L->n_theta)};
+    for (int i = 0; i < (whole ? 1 : 2) && s == CUBLAS_STATUS_SUCCESS; ++i) {
         const size_t j = (size_t)first[i];
         s = cublasGemmStridedBatchedEx(ctx->cublas, CUBLAS_OP_N, CUBLAS_OP_N, L->K_pad, (int)(2 * nb), R2, &one,
                                        (const uint16_t*)L->d_that + j * R2 * L->K_pad, CUDA_R_16BF, L->K_pad,
@@ -1064,13 +1072,16 @@ int prescore_rows(tm_ctx* ctx, cudaStream_t st, Library* const* libs, int n_libs
             }
             CUtensorMap emap, omap;
             const int ne = even_slots(n_theta), box_rows = (ne + 15) & ~15;   // (as many odd slots, or one less)
-            int rc = g_tensor_map(ctx, tb.g, (int)L->K, L->K_pad, nb, 0, ne, box_rows, &emap);
-            if (!rc)
+            const bool whole = whole_slots(L, nb);                 // (then one map serves both)
+            int rc = g_tensor_map(ctx, tb.g, (int)L->K, L->K_pad, nb, 0, whole ? tmgb::dense_slots() : ne, box_rows, &emap);
+            if (!rc && whole) omap = emap;
+            else if (!rc)
                 rc = g_tensor_map(ctx, tb.g, (int)L->K, L->K_pad, nb, tmgb::dense_slots() / 2, odd_slots(n_theta), box_rows,
                                   &omap);
             if (rc) return rc;
             tmgb::DenseCall dc{};
             dc.box_rows = box_rows;
+            dc.odd_slot = whole ? tmgb::dense_slots() / 2 : 0;
             dc.n = nb;
             dc.p0 = b0;
             dc.n_theta = n_theta;

@@ -289,6 +289,7 @@ struct DenseCall {
     int n_theta;
     int K;                     // templates of the library
     const void* basis;         // [2][96][192] bf16, K-major (dense_basis_rows x dense_basis_cols)
+    int odd_slot;              // first odd slot in omap
     int box_rows;              // slots of a part, a multiple of 16 (the tensor maps' boxes)
     const uint32_t* mask;      // [rows][words] templates to score (pre-filter) or null (all)
     int words;
