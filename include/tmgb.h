@@ -219,6 +219,12 @@ int tm_library_prepare_host(const tm_library_desc* desc, tm_library_info* info, 
 int tm_library_bound_entries_host(const tm_library_desc* desc, int32_t* n_words, int64_t* n_entries,
                                   int32_t* order, int32_t* word_start, int32_t* entries);
 
+/* Block sizes (threads) the kernel that scores templates behind their bounds can be launched
+ * with for libraries of n_rad distinct radii, n_theta angles and top_n results: *n_shapes of
+ * them in threads[3], 0 where the sparse kernel serves the call.  Needs no device. */
+int tm_score_shapes_host(int32_t n_rad, int32_t n_theta, int32_t top_n, int32_t* threads,
+                         int32_t* n_shapes);
+
 /* Stage 1 (Section 2.2, Fig. 2 (a)-(c)): gamma/subtract and bilinear polar resampling.
  * frames_dev [n][H][W] (TM_DTYPE_U16 or TM_DTYPE_F32, row-major, contiguous);
  * centres_dev [n][2] float (cx, cy) per pattern, finite, or NULL to use params->cx/cy for

@@ -59,11 +59,10 @@ __device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
 }
 
 // Largest block: 64 registers a thread hold up to 12 accumulators a lane, else 128.
-template <int NBMAX, int LAYOUT>
-constexpr int max_threads() { return NBMAX <= 12 ? 1024 : 512; }
+constexpr int max_threads(int nb_max) { return nb_max <= 12 ? 1024 : 512; }
 
 template <int NBMAX, int LAYOUT>
-__global__ void __launch_bounds__((max_threads<NBMAX, LAYOUT>()), 1)
+__global__ void __launch_bounds__(max_threads(NBMAX), 1)
 score_kernel(const ScoreCall c) {
     extern __shared__ __align__(16) float smem[];
     const SparseLib& L = c.lib;
@@ -429,40 +428,61 @@ score_kernel(const ScoreCall c) {
     if (c.work && lane == 0 && work) atomicAdd(c.work, work);
 }
 
-// Shared memory of the rows and lists (0: unsupported), the layout (wrap-free while two CTAs fit an
-// SM, else wrapped) and its pitch.  Not the dual layout: its halved loads gain less than its
-// shared memory costs in resident warps (FCC library, 16384 patterns with pre-filter: bounds and
-// scores 2.94 ms, wrap-free 2.60 ms).
-size_t score_smem(int n_rad, int n_theta, int top_n, int warps, int* layout, int* pitch) {
-    if (n_theta < 1 || n_theta > 1024 || top_n < 1 || top_n > TM_MAX_TOPN || n_rad < 1) return 0;
+// Accumulators a lane for n_theta shifts: the instantiation that serves them.
+int nb_max(int n_theta) {
+    const int nb = (n_theta + 31) / 32;
+    return nb <= 6 ? 6 : nb <= 12 ? 12 : nb <= 24 ? 24 : 32;
+}
+
+// Shared memory of the rows (row pitch `pitch`), the pool and the lists of `warps` warps.
+size_t score_smem(int n_rad, int pitch, int top_n, int warps) {
+    return (size_t)n_rad * pitch * 4 + 8 + (size_t)top_n * 8 + (size_t)warps * top_n * 12;
+}
+constexpr size_t kMaxSmem = 227 * 1024 - 2560;             // (the rest: the kernel's static arrays)
+
+// The row layout (wrap-free while two CTAs fit an SM, else wrapped) and its pitch; false where the
+// largest block's lists do not fit beside the rows.  Chosen once per call, for the largest block of
+// the instantiation, so every smaller block fits as well.  Not the dual layout: its halved loads gain
+// less than its shared memory costs in resident warps (FCC library, 16384 patterns with pre-filter:
+// bounds and scores 2.94 ms, wrap-free 2.60 ms).
+bool score_layout(int n_rad, int n_theta, int top_n, int* layout, int* pitch) {
+    if (n_theta < 1 || n_theta > 1024 || top_n < 1 || top_n > TM_MAX_TOPN || n_rad < 1) return false;
+    const int warps = max_threads(nb_max(n_theta)) / 32;
     const int order[2] = {TM_LAYOUT_WF, TM_LAYOUT_WRAP};
-    const size_t limit[2] = {113 * 1024, 227 * 1024};
+    const size_t limit[2] = {113 * 1024 - 2560, kMaxSmem};
     for (int i = 0; i < 2; ++i) {
         const int pch = sparse_pitch(n_theta, order[i]);
         if (order[i] == TM_LAYOUT_WF && (size_t)n_rad * pch > 65535) continue;   // 16-bit offsets
-        const size_t b = (size_t)n_rad * pch * 4 + 8 + (size_t)top_n * 8 + (size_t)warps * top_n * 12;
-        if (b + 2560 <= limit[i]) {
+        if (score_smem(n_rad, pch, top_n, warps) <= limit[i]) {
             *layout = order[i];
             *pitch = pch;
-            return b;
+            return true;
         }
     }
-    return 0;
+    return false;
+}
+
+int block_sizes(int n_rad, int n_theta, int pitch, int top_n, int threads[3]) {
+    int n = 0;
+    for (int t : {256, 512, 1024})
+        if (t <= max_threads(nb_max(n_theta)) && score_smem(n_rad, pitch, top_n, t / 32) <= kMaxSmem)
+            threads[n++] = t;
+    return n;
 }
 
 template <int NBMAX, int LAYOUT>
-cudaError_t launch_nb(const ScoreCall& call, int num_sms, cudaStream_t st) {
-    ScoreCall c = call;
+cudaError_t launch_nb(const ScoreCall& c, int num_sms, cudaStream_t st) {
     // Block size: with at most two patterns per SM, as many warps on each as fit; else the smallest
     // block that fills the SM's registers (blocks run their phases out of step).
     int threads = 0, per_sm = 0;
     size_t smem = 0;
     const int64_t share = (c.n + num_sms - 1) / num_sms;
-    for (int t : {256, 512, 1024}) {
-        if (t > max_threads<NBMAX, LAYOUT>()) break;
-        int layout, pitch, b = 0;
-        const size_t sm = score_smem(c.lib.n_rad, c.n_theta, c.top_n, t / 32, &layout, &pitch);
-        if (!sm || layout != LAYOUT) continue;
+    int sizes[3];
+    const int n_sizes = block_sizes(c.lib.n_rad, c.n_theta, c.pitch, c.top_n, sizes);
+    for (int i = 0; i < n_sizes; ++i) {
+        const int t = sizes[i];
+        int b = 0;
+        const size_t sm = score_smem(c.lib.n_rad, c.pitch, c.top_n, t / 32);
         const cudaError_t e = kernel_occupancy((const void*)score_kernel<NBMAX, LAYOUT>, t, sm, &b);
         if (e != cudaSuccess) return e;
         const int64_t used = std::min<int64_t>(b, share);
@@ -470,7 +490,6 @@ cudaError_t launch_nb(const ScoreCall& call, int num_sms, cudaStream_t st) {
             threads = t;
             per_sm = b;
             smem = sm;
-            c.pitch = pitch;
         }
     }
     if (!threads) return cudaErrorInvalidConfiguration;
@@ -482,26 +501,32 @@ cudaError_t launch_nb(const ScoreCall& call, int num_sms, cudaStream_t st) {
 
 }  // namespace
 
+// Block sizes that can take the call (0: the sparse kernel serves it).
+int score_shapes(int n_rad, int n_theta, int top_n, int threads[3]) {
+    int layout, pitch;
+    return score_layout(n_rad, n_theta, top_n, &layout, &pitch) ? block_sizes(n_rad, n_theta, pitch, top_n, threads) : 0;
+}
+
 bool score_supported(int n_rad, int n_theta, int top_n) {
     int layout, pitch;
-    return score_smem(n_rad, n_theta, top_n, kMaxWarps, &layout, &pitch) != 0;
+    return score_layout(n_rad, n_theta, top_n, &layout, &pitch);
 }
 
 cudaError_t launch_score(const ScoreCall& call, int num_sms, cudaStream_t st) {
     if (call.n <= 0) return cudaSuccess;
-    const ScoreCall& c = call;
-    int layout = TM_LAYOUT_WRAP, pitch = 0;
-    if (!score_smem(c.lib.n_rad, c.n_theta, c.top_n, kMaxWarps, &layout, &pitch)) return cudaErrorInvalidValue;
-    const int nb = (c.n_theta + 31) / 32;
+    ScoreCall c = call;
+    int layout = TM_LAYOUT_WRAP;
+    if (!score_layout(c.lib.n_rad, c.n_theta, c.top_n, &layout, &c.pitch)) return cudaErrorInvalidValue;
+    const int nb = nb_max(c.n_theta);
     if (layout == TM_LAYOUT_WF) {
-        if (nb <= 6) return launch_nb<6, TM_LAYOUT_WF>(c, num_sms, st);
-        if (nb <= 12) return launch_nb<12, TM_LAYOUT_WF>(c, num_sms, st);
-        if (nb <= 24) return launch_nb<24, TM_LAYOUT_WF>(c, num_sms, st);
+        if (nb == 6) return launch_nb<6, TM_LAYOUT_WF>(c, num_sms, st);
+        if (nb == 12) return launch_nb<12, TM_LAYOUT_WF>(c, num_sms, st);
+        if (nb == 24) return launch_nb<24, TM_LAYOUT_WF>(c, num_sms, st);
         return launch_nb<32, TM_LAYOUT_WF>(c, num_sms, st);
     }
-    if (nb <= 6) return launch_nb<6, TM_LAYOUT_WRAP>(c, num_sms, st);
-    if (nb <= 12) return launch_nb<12, TM_LAYOUT_WRAP>(c, num_sms, st);
-    if (nb <= 24) return launch_nb<24, TM_LAYOUT_WRAP>(c, num_sms, st);
+    if (nb == 6) return launch_nb<6, TM_LAYOUT_WRAP>(c, num_sms, st);
+    if (nb == 12) return launch_nb<12, TM_LAYOUT_WRAP>(c, num_sms, st);
+    if (nb == 24) return launch_nb<24, TM_LAYOUT_WRAP>(c, num_sms, st);
     return launch_nb<32, TM_LAYOUT_WRAP>(c, num_sms, st);
 }
 

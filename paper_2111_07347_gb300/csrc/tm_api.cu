@@ -1695,6 +1695,12 @@ int tm_library_bound_entries_host(const tm_library_desc* desc, int32_t* n_words,
     return TM_OK;
 }
 
+int tm_score_shapes_host(int32_t n_rad, int32_t n_theta, int32_t top_n, int32_t* threads, int32_t* n_shapes) {
+    if (!threads || !n_shapes) return fail(TM_ERR_INVALID_ARG, "tm_score_shapes_host: NULL output");
+    *n_shapes = tmgb::score_shapes(n_rad, n_theta, top_n, threads);
+    return TM_OK;
+}
+
 int tm_library_export(tm_ctx* ctx, int lib_id, int64_t* offsets, int32_t* r, int32_t* t, float* intensity,
                       float* norm, int32_t* order) {
     if (!ctx) return fail(TM_ERR_INVALID_ARG, "tm_library_export: ctx is NULL");

@@ -272,6 +272,8 @@ struct ScoreCall {
     int test_stall;
 };
 bool score_supported(int n_rad, int n_theta, int top_n);
+// Block sizes launch_score chooses from, returned count (0: not supported).
+int score_shapes(int n_rad, int n_theta, int top_n, int threads[3]);
 cudaError_t launch_score(const ScoreCall& c, int num_sms, cudaStream_t st);
 
 // ------------------------------------------------------------------ BF16 tensor-core path

@@ -121,6 +121,8 @@ _SIGS = {
                                                _P, _P, _P, _P, _P, _P, _P, _P]),
     "tm_library_bound_entries_host": (ctypes.c_int, [ctypes.POINTER(tm_library_desc), ctypes.POINTER(ctypes.c_int32),
                                                      ctypes.POINTER(ctypes.c_int64), _P, _P, _P]),
+    "tm_score_shapes_host": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
+                                            ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),
     "tm_polar_transform": (ctypes.c_int, [_P, ctypes.POINTER(tm_index_params), _P, ctypes.c_int32, ctypes.c_int64,
                                           ctypes.c_int32, ctypes.c_int32, _P, ctypes.c_int32, ctypes.c_int32,
                                           ctypes.c_double, _P, _P, _P, _P]),
@@ -272,6 +274,13 @@ def tm_library_bound_entries_host(ts, n_r: int, n_theta: int, dr: float = 1.0, m
                                                    out["order"].ctypes.data, out["word_start"].ctypes.data,
                                                    out["entries"].ctypes.data if ne.value else None))
     return out
+
+
+def tm_score_shapes_host(n_rad: int, n_theta: int, top_n: int) -> list:
+    """Block sizes the score kernel can be launched with (no GPU; empty: the sparse kernel serves the call)."""
+    threads, n = (ctypes.c_int32 * 3)(), ctypes.c_int32(0)
+    _check(library().tm_score_shapes_host(n_rad, n_theta, top_n, threads, ctypes.byref(n)))
+    return list(threads[:n.value])
 
 
 def _alloc_export(info):
