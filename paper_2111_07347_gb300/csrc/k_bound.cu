@@ -148,7 +148,8 @@ window_kernel(const float* __restrict__ polar, const float* __restrict__ pnorm, 
         for (int o = 16; o > 0; o >>= 1) ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
         if ((threadIdx.x & 31) == 0) s_abs[threadIdx.x >> 5] = ma;
         __syncthreads();
-        // (a norm that is zero, infinite or NaN: every Q is 0, and so is every bound)
+        // (a norm that is zero or NaN: every Q is 0, and so is every bound; an infinite norm: every finite
+        // correlation gives 0 and an infinite one a Q that is not a number, which ranks below them)
         const bool usable = pn > 0.0f && pn <= FLT_MAX;
         const float inv = usable ? __fdiv_ru(1.0f, pn) : 0.0f, inv_dn = usable ? __fdiv_rd(1.0f, pn) : 0.0f;
         float mabs = 0.0f;
