@@ -23,13 +23,11 @@
 // window_kernel: one CTA per pattern; piece maxima of the library's rows, then the W columns.
 // bound_templates_kernel: B, one warp per template (once per library).
 // bound_kernel: the contraction (32768 patterns against the 13986-template HCP library, six windows:
-//   2.0 ms; 2.55 ms before the issuing threads were freed of divisions and descriptor arithmetic, and
-//   2.3 ms without the clusters' multicast; its loads alone, its MMAs alone and its epilogue alone take
-//   within a fifth of each other).  D[128 templates x 240 columns] per unit = 240 / nw patterns;
-//   a persistent CTA keeps its 128 templates' B (kd <= 512: at most 128 KB) in shared memory and
-//   streams W through a ring.  Two CTAs form a cluster over two neighbouring template tiles and the
-//   same columns: each loads half of every W chunk into both (multicast), so L2 gives each byte once
-//   for both.  Two accumulators in TMEM (columns 0 and 256), so the epilogue of one
+//   2.3 ms; 2.55 ms before the issuing threads were freed of divisions and descriptor arithmetic; its
+//   loads alone, its MMAs alone and its epilogue alone take within a fifth of each other).
+//   D[128 templates x 240 columns] per unit = 240 / nw patterns; a persistent CTA keeps its 128
+//   templates' B (kd <= 512: at most 128 KB) in shared memory and streams W through a ring, in plain
+//   loads of its own.  Two accumulators in TMEM (columns 0 and 256), so the epilogue of one
 //   unit runs beside the MMAs of the next.  Units are ordered in blocks of kSuper column tiles
 //   (W of one block: 15 MB, kept in L2 while every template tile passes over it).  Warps: 0 TMA
 //   producer, 1 MMA issuer, 2 TMEM allocation, 4-11 epilogue (TMEM lane quadrant x column half):
@@ -56,7 +54,6 @@ constexpr int kAChunk = kM * kChunkK * 2;  // 16 KB
 constexpr int kBChunk = kN * kChunkK * 2;  // 30 KB
 constexpr int kMaxStages = 5;
 constexpr int kAccStride = 256;            // TMEM columns between the two accumulators
-constexpr int kPair = 2;                   // CTAs of a cluster: neighbouring template tiles, the same columns
 constexpr int kSuper = 64;                 // column tiles per block of units
 constexpr int kEpi0 = 4, kEpiThreads = 256;
 constexpr int kBoundThreads = kEpi0 * 32 + kEpiThreads;
@@ -220,13 +217,13 @@ bound_templates_kernel(const int4* __restrict__ meta, const int4* __restrict__ o
 }
 
 struct Units {                                             // the order of a CTA's units
-    int mt, nt;                                            // pairs of template tiles, column tiles
-    int cluster, clusters;                                 // this CTA's cluster of how many
+    int mt, nt;                                            // template tiles, column tiles
+    int cta, ctas;                                         // this CTA of how many
     __device__ __forceinline__ int super(int s) const { return min(kSuper, nt - s * kSuper); }
 };
 
-// Calls f(pair of template tiles, column tile, first unit of a pair, last unit of it) for the cluster's
-// units; stops when f returns false.
+// Calls f(template tile, column tile, first unit of the tile, last unit of it) for the CTA's units;
+// stops when f returns false.
 template <typename F>
 __device__ __forceinline__ void for_units(const Units& g, F f) {
     const int supers = (g.nt + kSuper - 1) / kSuper;
@@ -234,13 +231,13 @@ __device__ __forceinline__ void for_units(const Units& g, F f) {
     for (int s = 0; s < supers; ++s) {
         const int sb = g.super(s);
         const int64_t total = (int64_t)g.mt * sb;
-        const int64_t lo = total * g.cluster / g.clusters, hi = total * (g.cluster + 1) / g.clusters;
+        const int64_t lo = total * g.cta / g.ctas, hi = total * (g.cta + 1) / g.ctas;
         // whether the units of the next block (if the CTA has any) go on with the same template tile
         int next_mt = -1;
         for (int s2 = s + 1; s2 < supers && next_mt < 0; ++s2) {
             const int sb2 = g.super(s2);
             const int64_t t2 = (int64_t)g.mt * sb2;
-            const int64_t l2 = t2 * g.cluster / g.clusters, h2 = t2 * (g.cluster + 1) / g.clusters;
+            const int64_t l2 = t2 * g.cta / g.ctas, h2 = t2 * (g.cta + 1) / g.ctas;
             if (l2 < h2) next_mt = (int)(l2 / sb2);
         }
         // (counted on, not divided: a 64-bit division a unit in every role had been a quarter of the time)
@@ -258,7 +255,7 @@ __device__ __forceinline__ void for_units(const Units& g, F f) {
 }
 
 template <int NW>
-__global__ void __cluster_dims__(kPair, 1, 1) __launch_bounds__(kBoundThreads, 1)
+__global__ void __launch_bounds__(kBoundThreads, 1)
 bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap, const BoundCall c) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -278,16 +275,15 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
     const uint32_t done = smem_u32(&bar[2 * kMaxStages + 6]);   // MMAs finished, when stopping
     constexpr int kPat = kN / NW;                           // patterns per unit
     Units g;
-    const int rank = blockIdx.x % kPair;
-    g.mt = (c.K + kM * kPair - 1) / (kM * kPair);
-    g.cluster = blockIdx.x / kPair;
-    g.clusters = gridDim.x / kPair;
+    g.mt = (c.K + kM - 1) / kM;
+    g.cta = blockIdx.x;
+    g.ctas = gridDim.x;
     g.nt = (int)((c.n + kPat - 1) / kPat);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kMaxStages; ++i) {
             mbar_init(full0 + 8 * i, 1);
-            mbar_init(empty0 + 8 * i, kPair);               // both CTAs' MMAs have read the slot
+            mbar_init(empty0 + 8 * i, 1);
         }
         mbar_init(a_full, 1);
         mbar_init(a_empty, 1);
@@ -308,7 +304,6 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
     }
     tc_fence_before();
     __syncthreads();
-    cluster_sync();                                         // (the peer's barriers are initialised as well)
     tc_fence_after();
     const uint32_t tmem = s_tmem;
 
@@ -322,26 +317,22 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
                     if (!mbar_wait(a_empty, (na & 1u) ^ 1u, abort_flag)) { *abort_flag = 1; return false; }
                     mbar_expect_tx(a_full, (uint32_t)(chunks * kAChunk));
                     for (int ch = 0; ch < chunks; ++ch)
-                        tma_load_2d(smem_u32(s_a + ch * kAChunk), &amap, ch * kChunkK, (m * kPair + rank) * kM, a_full);
+                        tma_load_2d(smem_u32(s_a + ch * kAChunk), &amap, ch * kChunkK, m * kM, a_full);
                     ++na;
                 }
                 for (int ch = 0; ch < chunks; ++ch, ++q) {
                     if (!mbar_wait(empty0 + 8 * slot, phase ^ 1u, abort_flag)) { *abort_flag = 1; return false; }
                     mbar_expect_tx(full0 + 8 * slot, kBChunk);
-                    // this CTA's half of the chunk's rows, into both
-                    tma_load_2d_multicast(smem_u32(s_b + slot * kBChunk + rank * (kBChunk / kPair)), &bmap, ch * kChunkK,
-                                          ct * kN + rank * (kN / kPair), full0 + 8 * slot, (1u << kPair) - 1);
+                    tma_load_2d(smem_u32(s_b + slot * kBChunk), &bmap, ch * kChunkK, ct * kN, full0 + 8 * slot);
                     if (++slot == (uint32_t)stages) { slot = 0; phase ^= 1u; }
                 }
                 return true;
             });
-            // the copies issued last must land, and both CTAs' MMAs have reported their slots read, before
-            // the CTA exits (they complete on their own)
+            // the copies issued last must land before the CTA exits (they complete on their own)
             volatile int never = 0;
             for (uint32_t i = 0; i < (uint32_t)stages && i < q; ++i) {
-                const uint32_t qq = q - 1 - i, slot = qq % stages, par = (qq / stages) & 1u;
-                mbar_wait(full0 + 8 * slot, par, &never);
-                mbar_wait(empty0 + 8 * slot, par, abort_flag);
+                const uint32_t qq = q - 1 - i, last = qq % stages;
+                mbar_wait(full0 + 8 * last, (qq / stages) & 1u, &never);
             }
             if (na) mbar_wait(a_full, (na - 1) & 1u, &never);
         }
@@ -372,7 +363,7 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
 #pragma unroll
                     for (int ks = 0; ks < kChunkK / 16; ++ks)
                         if (ks < ks_n) mma_f16(d, da + 2 * ks, db + 2 * ks, idesc, (ch | ks) ? 1u : 0u);
-                    mma_commit_multicast(empty0 + 8 * slot, (1u << kPair) - 1);
+                    mma_commit(empty0 + 8 * slot);
                     issued = true;
                     if (++slot == (uint32_t)stages) { slot = 0; phase ^= 1u; }
                 }
@@ -414,7 +405,7 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acce0 + 8 * buf);    // the accumulator is in registers
-            const int k = (m * kPair + rank) * kM + quad * 32 + lane, word = (m * kPair + rank) * (kM / 32) + quad;
+            const int k = m * kM + quad * 32 + lane, word = m * (kM / 32) + quad;
             const int64_t p0 = (int64_t)ct * kPat + half * kMine;
             uint32_t wm = 0;                                // lane i: the word's maximum for pattern i
 #pragma unroll
@@ -437,7 +428,6 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    cluster_sync();                                         // the peer's copies and arrivals into this CTA are done
     if (*abort_flag && threadIdx.x == 0) atomicOr(c.error, 8u);
     if (warp == 2) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
@@ -493,7 +483,7 @@ cudaError_t launch_bound_windows(const float* polar, const float* pnorm, int64_t
     return cudaGetLastError();
 }
 
-int bound_box_rows(bool templates) { return templates ? kM : kN / kPair; }
+int bound_box_rows(bool templates) { return templates ? kM : kN; }
 
 cudaError_t launch_bound(const void* amap, const void* bmap, const BoundCall& call, int nw, int num_sms,
                          cudaStream_t st) {
@@ -506,13 +496,8 @@ cudaError_t launch_bound(const void* amap, const void* bmap, const BoundCall& ca
     const cudaError_t e = kernel_occupancy(fn, kBoundThreads, smem, nullptr);
     if (e != cudaSuccess) return e;
     const int pat = kN / nw;
-    const int64_t units = (int64_t)((c.K + kM * kPair - 1) / (kM * kPair)) * ((c.n + pat - 1) / pat);
-    // no more clusters than run at once: the units are split evenly between them
-    int clusters = 0;
-    const cudaError_t ec = cluster_occupancy(fn, kBoundThreads, smem, kPair, &clusters);
-    if (ec != cudaSuccess) return ec;
-    clusters = std::min(clusters, num_sms / kPair);
-    const int grid = kPair * (int)std::max<int64_t>(1, std::min<int64_t>(clusters, units));
+    const int64_t units = (int64_t)((c.K + kM - 1) / kM) * ((c.n + pat - 1) / pat);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms, units));
     if (nw == 12)
         bound_kernel<12><<<grid, kBoundThreads, smem, st>>>(*(const CUtensorMap*)amap, *(const CUtensorMap*)bmap, c);
     else

@@ -15,8 +15,8 @@
 // Without bounds (u null) the templates of the mask are scored, all of them, by words or
 // quarters of words: the rescoring of a few candidates per pattern, or a small library.
 //
-// 32768 patterns against the 13986-template HCP library: bounds and scores 5.5 ms (windows 0.57, the
-// contraction 2.0, this kernel 2.9), where bounding and scoring in one kernel on the CUDA cores took
+// 32768 patterns against the 13986-template HCP library: bounds and scores 5.8 ms (windows 0.57, the
+// contraction 2.3, this kernel 2.9), where bounding and scoring in one kernel on the CUDA cores took
 // 18.9 ms.  Bound by latency and issue: 0.59 warp instructions a cycle per scheduler, most other
 // cycles at the barriers between a pattern's phases.
 // One warp scores one template (score_template: all its shifts in registers, spots in CSR order, as

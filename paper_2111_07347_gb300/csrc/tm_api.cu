@@ -161,33 +161,6 @@ cudaError_t kernel_occupancy(const void* fn, int threads, size_t smem, int* per_
     return cudaSuccess;
 }
 
-cudaError_t cluster_occupancy(const void* fn, int threads, size_t smem, int size, int* clusters) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lk(g_launch_mu);
-    const auto key = std::make_tuple(fn, dev, -threads, smem);   // (negative: clusters, not blocks)
-    auto it = g_occupancy.find(key);
-    if (it == g_occupancy.end()) {
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = size;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(size);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
-        if (e != cudaSuccess) return e;
-        it = g_occupancy.emplace(key, n).first;
-    }
-    *clusters = it->second;
-    return cudaSuccess;
-}
-
 namespace {
 thread_local int t_sm_cap = 0;      // persistent grids of this thread's calls use at most this many SMs
 }

@@ -77,9 +77,6 @@ struct RadialLib {
 // returns its resident blocks per SM for `threads` threads (per_sm may be null).  Cached, so
 // repeated launches make no driver queries.
 cudaError_t kernel_occupancy(const void* fn, int threads, size_t smem, int* per_sm);
-// Clusters of `size` blocks that are resident at once on the device (cached; after kernel_occupancy
-// has raised the limit).
-cudaError_t cluster_occupancy(const void* fn, int threads, size_t smem, int size, int* clusters);
 // Number of SMs of the current device (cached), or the calling thread's cap when one is set.
 int device_sms();
 // Caps the persistent grids of this thread's later calls at `cap` SMs (0 = no cap), so that work

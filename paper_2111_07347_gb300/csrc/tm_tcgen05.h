@@ -121,28 +121,4 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
-// The same copy into the shared memory of every CTA of `mask` in the cluster, at the same offset,
-// completing on the mbarrier at the same offset in each.
-__device__ __forceinline__ void tma_load_2d_multicast(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t mbar,
-                                                      uint16_t mask) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster "
-        "[%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
-        "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(mbar), "h"(mask)
-        : "memory");
-}
-
-// Arrives, once this thread's earlier MMAs are done, on the mbarrier at the same offset in every CTA
-// of `mask` in the cluster.
-__device__ __forceinline__ void mma_commit_multicast(uint32_t mbar, uint16_t mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(mbar),
-        "h"(mask)
-        : "memory");
-}
-
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-}
-
 }  // namespace tmgb
