@@ -99,10 +99,13 @@ struct Library {
     int32_t* d_rowmap = nullptr;   // [n_r] radius -> row among the distinct radii (-1: none)
     int R = 0, K_pad = 0;
     size_t that_bytes = 0;
-    // templates of the tensor-core bounds (k_bound.cu), built on first use: [K][pitch] FP16
+    // templates of the tensor-core bounds (k_bound.cu), built when the library is loaded (with a
+    // budget, on first use): [K][pitch] FP16 and, behind them, their order
+    bool boundable = false;        // whether the bounds take this library, and their shape
     tmgb::BoundShape bshape;
+    std::vector<int32_t> by_spots; // template indices, fewest spots first, ties by index
     void* d_bound = nullptr;
-    int4* d_border = nullptr;      // [32 words] the templates in the bounds' order, fewest spots first
+    int4* d_border = nullptr;      // [32 words] {first spot, spots | shifts << 16, norm bits, template}
     size_t bound_bytes = 0;
 };
 
@@ -205,6 +208,7 @@ struct tm_ctx {
         int64_t launches = 0, corr = 0, scored = 0;
     };
     std::map<std::string, GraphEntry> graphs;
+    size_t bound_refused = 0;      // ctx->used when the device last had no room for bound templates (0: never)
     uint64_t ws_gen = 1;           // bumped whenever a workspace buffer is reallocated
     bool capturing = false;
     // autotuned sparse-kernel shape per library signature (tm_autotune): block size and
@@ -518,6 +522,17 @@ int prepare_library(const tm_library_desc* d, Library* L, Prepared* P) {
         memcpy(&sb, &fs, 4);
         P->meta[k] = make_int4((int32_t)L->off[k], (int32_t)(cnt | ((int64_t)P->nshift[k] << 16)), nb, sb);
     }
+    // the order of the tensor-core bounds: a counting sort by spots
+    {
+        std::vector<int32_t> start(L->max_spots + 2, 0);
+        for (int64_t k = 0; k < L->K; ++k) ++start[L->off[k + 1] - L->off[k] + 1];
+        for (int c = 0; c <= L->max_spots; ++c) start[c + 1] += start[c];
+        L->by_spots.resize(L->K);
+        for (int64_t k = 0; k < L->K; ++k) L->by_spots[start[L->off[k + 1] - L->off[k]]++] = (int32_t)k;
+        // finer windows where templates of like weights compete: unit intensities, or many spots
+        const bool fine = L->unit || (int64_t)L->r.size() >= 20 * L->K;
+        L->boundable = L->nonneg && tmgb::bound_shape((int)std::max<size_t>(1, L->radii.size()), n_theta, fine, &L->bshape);
+    }
     // the bound entries again, templates ordered by spot count (descending, stable: the words
     // taken last are the cheapest) and each word's entries stored spot-major with its 32 lanes
     // adjacent, so the bound loop of a warp neither diverges much nor scatters its loads;
@@ -618,8 +633,7 @@ int build_library(tm_ctx* ctx, const tm_library_desc* d, Library* L) {
 void free_library(tm_ctx* ctx, Library* L) {
     void* ps[] = {L->d_off,    L->d_spot,  L->d_spot2, L->d_meta,  L->d_norm,   L->d_nshift, L->d_radial,
                   L->d_rnorm,  L->d_rt,    L->d_radii, L->d_bspot, L->d_that,   L->d_rowmap,
-                  L->d_smeta,  L->d_sperm, L->d_ellw,  L->d_ell,  L->d_bound,
-                  L->d_border};
+                  L->d_smeta,  L->d_sperm, L->d_ellw,  L->d_ell,  L->d_bound};
     for (void* p : ps)
         if (p) cudaFree(p);
     ctx->used -= std::min(ctx->used, L->bytes + L->that_bytes + L->bound_bytes);
@@ -838,61 +852,85 @@ int ensure_spectra(tm_ctx* ctx, Library* L, const SpectralTables& spec, cudaStre
     return TM_OK;
 }
 
-// Whether the library has the templates of the tensor-core bounds, built on the device the first
-// time it is asked (the call waits for the build, so that work on other streams can use them as
-// soon as it returns).  Not for libraries with negative intensities or more radii than the
-// contraction takes, nor while their memory is not to be had (the budget; a stream that is
-// being captured): such calls bound and score in the sparse kernel.
-bool ensure_bounds(tm_ctx* ctx, Library* L, cudaStream_t st) {
-    if (L->d_bound) return true;
-    const int n_rad = (int)std::max<size_t>(1, L->radii.size());
-    // finer windows where templates of like weights compete: unit intensities, or many spots
-    const bool fine = L->unit || (int64_t)L->r.size() >= 20 * L->K;
-    if (!L->nonneg || !tmgb::bound_shape(n_rad, L->n_theta, fine, &L->bshape)) return false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (ctx->capturing || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
+// A library of less templates is scored whole: the bounds' two launches and their latency cost more
+// than the scores they would save (300 templates of 24 spots, 256 patterns: 137 us with bounds, 83 us
+// without).
+constexpr int kBoundTemplates = 512;
+
+size_t bound_order_at(const Library* L) { return ((size_t)L->K * L->bshape.pitch * 2 + 255) & ~(size_t)255; }
+size_t bound_need(const Library* L) {
+    return bound_order_at(L) + (size_t)(L->K + 31) / 32 * 32 * sizeof(int4);
+}
+
+// The library's bound templates on the device; the call waits for the build, so that work on any
+// stream can use them as soon as it returns.
+bool build_bounds(tm_ctx* ctx, Library* L, cudaStream_t st) {
+    const std::string err = g_err;
+    const size_t bytes = bound_need(L);
+    void* p = nullptr;
+    if (dev_alloc(ctx, &p, bytes, "library bound templates")) {
+        g_err = err;                               // (such calls bound and score in the sparse kernel)
+        ctx->bound_refused = std::max<size_t>(1, ctx->used);
         return false;
     }
-    // the order of the bounds: by spot count, fewest first, ties by index
-    std::vector<int32_t> perm(L->K);
-    for (int64_t k = 0; k < L->K; ++k) perm[k] = (int32_t)k;
-    std::stable_sort(perm.begin(), perm.end(),
-                     [&](int32_t a, int32_t b) { return L->off[a + 1] - L->off[a] < L->off[b + 1] - L->off[b]; });
     std::vector<int4> order((L->K + 31) / 32 * 32, make_int4(0, 0, 0, -1));
     for (int64_t j = 0; j < L->K; ++j) {
-        const int32_t k = perm[j];
+        const int32_t k = L->by_spots[j];
         int32_t nb;
         memcpy(&nb, &L->norm[k], 4);
         order[j] = make_int4((int32_t)L->off[k],
                              (int32_t)((L->off[k + 1] - L->off[k]) | ((int64_t)(L->n_theta / L->order[k]) << 16)), nb, k);
     }
-    const size_t bytes = (size_t)L->K * L->bshape.pitch * 2, ob = order.size() * sizeof(int4);
-    void *b = nullptr, *o = nullptr;
-    const std::string err = g_err;
-    if (dev_alloc(ctx, &b, bytes, "library bound templates")) {
-        g_err = err;
-        return false;
-    }
-    if (dev_alloc(ctx, &o, ob, "library bound order")) {
-        g_err = err;
-        dev_free(ctx, b, bytes);
-        return false;
-    }
-    cudaError_t e = cudaMemcpyAsync(o, order.data(), ob, cudaMemcpyHostToDevice, st);
+    int4* o = (int4*)((char*)p + bound_order_at(L));
+    cudaError_t e = cudaMemcpyAsync(o, order.data(), order.size() * sizeof(int4), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
-        e = tmgb::launch_bound_templates(L->d_meta, (const int4*)o, L->d_spot, (int)L->K, L->n_theta, n_rad, L->bshape,
-                                         b, st);
+        e = tmgb::launch_bound_templates(L->d_meta, o, L->d_spot, (int)L->K, L->n_theta,
+                                         (int)std::max<size_t>(1, L->radii.size()), L->bshape, p, st);
     const cudaError_t e2 = cudaStreamSynchronize(st);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         cudaGetLastError();
-        dev_free(ctx, b, bytes);
-        dev_free(ctx, o, ob);
+        dev_free(ctx, p, bytes);
         return false;
     }
-    L->d_bound = b;
-    L->d_border = (int4*)o;
-    L->bound_bytes = bytes + ob;
+    L->d_bound = p;
+    L->d_border = o;
+    L->bound_bytes = bytes;
+    return true;
+}
+
+// Whether every library of a call (null: not needed) has its bound templates; missing ones are
+// built, all of them or none.  Not for libraries that the bounds do not take, nor where the budget
+// has no room for all of them, nor on a stream that is being captured.  A device without room is
+// asked again once the context has given memory back.
+bool ensure_bounds(tm_ctx* ctx, Library* const* libs, int n_libs, cudaStream_t st) {
+    size_t need = 0;
+    for (int i = 0; i < n_libs; ++i) {
+        if (libs[i] && !libs[i]->boundable) return false;
+        if (libs[i] && !libs[i]->d_bound) need += bound_need(libs[i]);   // (a library named twice counts twice)
+    }
+    if (!need) return true;
+    if (ctx->budget && ctx->used + need > ctx->budget) return false;
+    if (ctx->bound_refused && ctx->used >= ctx->bound_refused) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (ctx->capturing || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    bool built[TM_MAX_LIBS] = {};
+    for (int i = 0; i < n_libs; ++i) {
+        if (!libs[i] || libs[i]->d_bound) continue;
+        built[i] = build_bounds(ctx, libs[i], st);
+        if (built[i]) continue;
+        for (int j = 0; j < i; ++j)
+            if (built[j]) {
+                dev_free(ctx, libs[j]->d_bound, libs[j]->bound_bytes);
+                libs[j]->d_bound = nullptr;
+                libs[j]->d_border = nullptr;
+                libs[j]->bound_bytes = 0;
+            }
+        return false;
+    }
+    ctx->bound_refused = 0;
     return true;
 }
 
@@ -1580,6 +1618,9 @@ int tm_load_library(tm_ctx* ctx, const tm_library_desc* desc, int* lib_id) {
         free_library(ctx, L.get());
         return rc;
     }
+    // the bound templates at once, so that the first indexing call need not wait for them; with a budget
+    // they are left to a call that uses them, and later loads find the room
+    if (!ctx->budget && L->boundable && L->K >= kBoundTemplates) build_bounds(ctx, L.get(), nullptr);
     const int id = ctx->next_id++;
     ctx->libs.emplace(id, std::move(L));
     *lib_id = id;
@@ -1845,16 +1886,15 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
     // FP32 path: bounds of every template on the tensor cores, then the exact scores of the few
     // templates they leave (k_bound.cu, k_score.cu), where every library has them; else the sparse
     // kernel bounds and scores in one.  BF16 path: the candidates are scored by the score kernel.
-    // A library of less than 512 templates is scored whole: the bounds' two launches and their
-    // latency cost more than the scores they would save (300 templates of 24 spots, 256 patterns:
-    // 137 us with bounds, 83 us without).
-    bool bounds = !bf16, scores = true;
+    bool scores = true;
     bool whole[TM_MAX_LIBS];
+    Library* bounded[TM_MAX_LIBS];
     for (int i = 0; i < n_libs; ++i) {
         scores = scores && tmgb::score_supported((int)std::max<size_t>(1, libs[i]->radii.size()), n_theta, N);
-        whole[i] = libs[i]->K < 512;
-        bounds = bounds && scores && (whole[i] || ensure_bounds(ctx, libs[i], st));
+        whole[i] = libs[i]->K < kBoundTemplates;
+        bounded[i] = whole[i] ? nullptr : libs[i];
     }
+    const bool bounds = !bf16 && scores && ensure_bounds(ctx, bounded, n_libs, st);
 
     // chunk size from a per-pattern workspace estimate (<= 4 GiB of workspace)
     size_t per = (size_t)n_r * n_theta * 4 + 4 + (size_t)n_r * 4 + 4;
