@@ -269,10 +269,13 @@ int tm_correlate(tm_ctx* ctx, int lib_id, const float* polar_dev, const float* n
 int tm_prescore(tm_ctx* ctx, int lib_id, const float* polar_dev, const float* norm_dev,
                 const float* radial_dev, int64_t n, double fraction, float* score_dev, void* stream);
 
-/* Autotune the FP32 sparse kernel for a set of libraries: time its shapes -- block size (128,
- * 256, 512 threads; by default 256, or 512 where the rows leave an SM two blocks or one) x templates seeded per warp for the pruned top-N (4, 8, 16;
- * default 8: the templates of highest bound are scored first, so that the top-N threshold
- * the others are pruned against starts high) on the first min(n, 2048) frames, then the best
+/* Autotune the FP32 sparse kernel for a set of libraries.  It serves the top-N calls that the
+ * bounds on the tensor cores do not take (more than 56 radii, negative intensities, no room for
+ * the bound templates); the others do not use the shape.  Times the kernel's shapes -- block
+ * size (128, 256, 512 threads; by default 256, or 512 where the rows leave an SM two blocks or
+ * one) x templates seeded per warp for the pruned top-N (4, 8, 16; default 8: the templates
+ * of highest bound are scored first, so that the top-N threshold the others are pruned
+ * against starts high) on the first min(n, 2048) frames, then the best
  * of these against its block size with 4 patterns per CTA bounded together (default 1) and
  * each seed count on the first min(n, 16384) -- with these parameters, keep the fastest for
  * later calls on libraries of the same shapes (template count, spot count, radii, n_theta)

@@ -1894,7 +1894,8 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
         whole[i] = libs[i]->K < kBoundTemplates;
         bounded[i] = whole[i] ? nullptr : libs[i];
     }
-    const bool bounds = !bf16 && scores && ensure_bounds(ctx, bounded, n_libs, st);
+    // (while shapes of the sparse kernel are timed, it serves the call)
+    const bool bounds = !bf16 && scores && !ctx->tune_override.threads && ensure_bounds(ctx, bounded, n_libs, st);
 
     // chunk size from a per-pattern workspace estimate (<= 4 GiB of workspace)
     size_t per = (size_t)n_r * n_theta * 4 + 4 + (size_t)n_r * 4 + 4;
