@@ -13,10 +13,11 @@
 // W[(a, j); h] / |P|, and U[k, p] = max_h (B W)[k, (p, h)].
 //
 // Why U is a bound of Q as the exact kernels compute it: W is FP16 rounded up and I >= 0.  B is FP16
-// rounded to nearest, which changes the sum by at most 2^-11 sum|I| / |T| max|P'| / |P|; the products
-// are exact in FP32 and their sum is off by less than 512 * 2^-22 of the same; the exact sum by at
-// most (2 spots + 40) 2^-24 of it.  The last entry of the contraction adds all three (factors
-// rounded up); the result is raised by 2^-18 of itself for the rounding of Q's division, and
+// rounded to nearest, which changes an entry by at most 2^-11 of itself or, below 2^-14 (subnormal),
+// by 2^-25, so the sum by at most (2^-11 sum|I| / |T| + 2^-25 entries) max|P'| / |P|; the products
+// are exact in FP32 and their sum is off by less than 512 * 2^-22 of sum|I| / |T| max|P'| / |P|; the
+// exact sum by at most (2 spots + 40) 2^-24 of that.  The last entry of the contraction adds all of it
+// (factors rounded up); the result is raised by 2^-18 of itself for the rounding of Q's division, and
 // rounded up to FP16.  So a template with U below the N-th best Q found so far can be left out
 // without changing the result.
 //
@@ -208,9 +209,11 @@ bound_templates_kernel(const int4* __restrict__ meta, const int4* __restrict__ o
             *e += __fdiv_rn(__int_as_float(sp.y), tn);
         }
         // the margins' factor: ((2 spots + 40) 2^-24 + 2^-11 + 2^-13) sum|I| / |T| (2^-22 more for the
-        // FP32 sums of B)
+        // FP32 sums of B), and 2^-25 for every entry that holds a spot
         const float rel = (2.0f * (float)cnt + 40.0f) * 5.9604645e-8f + 6.1059e-4f;
-        row[n_rad * s.nch] = __fmul_ru(kMarginScale, __fdiv_ru(__fmul_ru(rel, __int_as_float(m.w)), tn));
+        const float tiny = (float)min(cnt, n_rad * s.nch) * 2.9802322e-8f;
+        row[n_rad * s.nch] =
+            __fmul_ru(kMarginScale, __fadd_ru(__fdiv_ru(__fmul_ru(rel, __int_as_float(m.w)), tn), tiny));
     }
     __syncwarp();
     for (int i = lane; i < s.pitch; i += 32) out[(size_t)k * s.pitch + i] = i == n_rad * s.nch ? __float2half_ru(row[i]) : __float2half_rn(row[i]);
