@@ -125,13 +125,14 @@ typedef struct tm_index_params {
  * is on. */
 #define TM_INDEX_GRAPH 1
 
-/* tm_index_params.reserved flag for tests of the failure path: the BF16 tensor-core kernel's
- * MMA issuer issues nothing, so its producer and epilogue waits run out (about 1 s each);
- * the kernel records the timeout in the context's device error word, stops its roles,
- * frees its tensor memory and returns.  The FP32 sparse kernel's row staging (bulk copies,
- * for n_theta a multiple of 4 outside the dual row layout) expects 16 bytes more than its
- * copies bring, so its wait runs out (about 1 s, then 1 s more for the copies); it records
- * the timeout and returns.  tm_check then reports TM_ERR_TIMEOUT; the call's hits are
+/* tm_index_params.reserved flag for tests of the failure path: the MMA issuers of the two
+ * tensor-core kernels (BF16 pre-score, FP32 bounds) issue nothing, so their producer and
+ * epilogue waits run out (about 1 s each); the kernel records the timeout in the context's
+ * device error word, stops its roles, frees its tensor memory and returns.  The row staging
+ * of the FP32 kernels that score templates (bulk copies, for n_theta a multiple of 4; in
+ * the sparse kernel outside its dual row layout) expects 16 bytes more than its copies
+ * bring, so its wait runs out (about 1 s, then 1 s more for the copies); it records the
+ * timeout and returns.  tm_check then reports TM_ERR_TIMEOUT; the call's hits are
  * meaningless; the context stays usable. */
 #define TM_INDEX_TEST_STALL 2
 

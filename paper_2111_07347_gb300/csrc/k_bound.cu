@@ -341,7 +341,7 @@ bound_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ C
         }
     } else if (warp == 1) {
         // ================================================================ MMA issuer
-        if (lane == 0) {
+        if (lane == 0 && !c.stall) {
             const uint32_t idesc = idesc_f16(kM, kN);
             const uint64_t a_desc = sdesc_kmajor(smem_u32(s_a)), b_desc = sdesc_kmajor(smem_u32(s_b));
             uint32_t na = 0, tt = 0, slot = 0, phase = 0;

@@ -2035,6 +2035,7 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
                     bc.u = bu;
                     bc.wmax = bmax;
                     bc.error = ctx->d_error;
+                    bc.stall = (params->reserved & TM_INDEX_TEST_STALL) ? 1 : 0;
                     TM_CUDA(tmgb::launch_bound(&amap, &bmap, bc, bs.nw, sms, st), "tm_index_patterns: bounds");
                     sc.order = L->d_border;
                     sc.u = bu;

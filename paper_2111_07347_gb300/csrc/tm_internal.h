@@ -240,6 +240,7 @@ struct BoundCall {
     unsigned short* u;         // [n][32 words] FP16 as order-preserving keys
     unsigned short* wmax;      // [n][words] keys: the largest of each 32 templates
     unsigned* error;           // device word: bit 8 = a bounded wait timed out
+    int stall;                 // test: issue no MMAs, so every wait runs out
     int stages;                // set by launch_bound
 };
 int bound_box_rows(bool templates);        // rows of the tensor maps' boxes (64 halves wide, 128-byte swizzle)
