@@ -37,10 +37,10 @@ __global__ void refine_kernel(const RefineCall c) {
         const int64_t p = rest / c.top_n;
         const int j = (int)(rest - p * c.top_n);
         tm_hit* h = c.hits + (size_t)li * c.hits_lib_stride + (size_t)p * c.top_n + j;
-        const int k = h->template_index;
-        if (k < 0) continue;
-        const int s = h->shift;
+        const int k = h->template_index, s = h->shift;
         const RefineLib& L = c.lib[li];
+        // (no hit; or rows that a kernel which stopped on a wait never wrote)
+        if ((unsigned)k >= (unsigned)L.K || (unsigned)s >= (unsigned)c.n_theta) continue;
         const float d = __ldg(c.pnorm + p) * __ldg(L.norm + k);
         const float* P = c.polar + (size_t)p * c.n_r * c.n_theta;
         const int beg = __ldg(L.off + k), end = __ldg(L.off + k + 1);

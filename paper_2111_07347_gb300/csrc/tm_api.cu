@@ -2142,7 +2142,7 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
                 rc.top_n = N;
                 rc.n_libs = n_libs;
                 for (int i = 0; i < n_libs; ++i)
-                    rc.lib[i] = tmgb::RefineLib{libs[i]->d_off, libs[i]->d_rt, libs[i]->d_spot, libs[i]->d_norm};
+                    rc.lib[i] = tmgb::RefineLib{libs[i]->d_off, libs[i]->d_rt, libs[i]->d_spot, libs[i]->d_norm, (int)libs[i]->K};
                 rc.hits = out_dev + (size_t)c0 * N;
                 rc.hits_lib_stride = lib_stride;
                 TM_CUDA(tmgb::launch_refine(rc, sms, st), "tm_index_patterns: refine");

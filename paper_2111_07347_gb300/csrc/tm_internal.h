@@ -106,6 +106,7 @@ struct RefineLib {
     const int32_t* rt;         // [n_spots]  r | t << 16
     const int2* spot;          // [n_spots]  .y = intensity bits
     const float* norm;         // [K]
+    int K;
 };
 struct RefineCall {
     const float* polar;        // [n][n_r][n_theta]  (rows of the libraries' radii)

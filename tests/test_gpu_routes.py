@@ -112,3 +112,23 @@ def test_waits_run_out_and_the_context_goes_on(which, launches, bits):
     assert torch.equal(ctx.index(f, lid, top_n=5), want)
     ctx.check()
     ctx.close()
+
+
+def test_refinement_leaves_unwritten_rows_alone():
+    """A scoring kernel that stopped on a wait leaves rows of the caller's buffer as they were; the angle
+    refinement that follows reads no template through them."""
+    import torch
+    ts = synth.kinematic_library("hcp", step_deg=2.0)
+    f = _frames(ts, 8, 360, 87)
+    ctx = tmgb.Context(0)
+    lid = ctx.load_library(ts, 128, 360)
+    out = torch.full((1, 8, 5, 5), 0x7F7F7F7F, dtype=torch.int32, device="cuda")
+    kept = out.clone()
+    ctx.index(f, lid, top_n=5, refine=True, test_stall=True, out=out)
+    with pytest.raises(tmgb.TmError):
+        ctx.check()
+    assert torch.equal(out, kept)
+    ctx.index(f, lid, top_n=5, refine=True, out=out)
+    ctx.check()
+    assert (out[..., 0] >= 0).all()
+    ctx.close()
