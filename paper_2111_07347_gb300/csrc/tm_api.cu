@@ -1283,13 +1283,16 @@ int tm_frame_sum(tm_ctx* ctx, const void* frames_dev, int32_t dtype, int64_t n, 
         TM_CUDA(cudaMemsetAsync(sum_dev, 0, (size_t)H * W * sizeof(double), st), "tm_frame_sum: memset");
         return TM_OK;
     }
+    // partial sums of groups of frames; fewer groups where there is no room for them
     void* scratch = nullptr;
-    const size_t sb = tmgb::frame_sum_scratch_bytes(dtype, n, H, W, ctx->num_sms);
-    if (sb) {
-        int rc = workspace(ctx, st, "frame_sum_partials", sb, &scratch);
-        if (rc) return rc;
+    int groups = 1, rc = TM_OK;
+    for (bool few : {false, true}) {
+        groups = tmgb::frame_sum_groups(dtype, n, H, W, ctx->num_sms, few);
+        rc = groups > 1 ? workspace(ctx, st, "frame_sum_partials", (size_t)groups * H * W * sizeof(double), &scratch) : TM_OK;
+        if (rc != TM_ERR_OOM) break;
     }
-    TM_CUDA(tmgb::launch_frame_sum(frames_dev, dtype, n, H, W, accumulate ? 1 : 0, sum_dev, (double*)scratch,
+    if (rc) return rc;
+    TM_CUDA(tmgb::launch_frame_sum(frames_dev, dtype, n, H, W, accumulate ? 1 : 0, sum_dev, (double*)scratch, groups,
                                    ctx->num_sms, st),
             "tm_frame_sum: launch");
     return TM_OK;

@@ -152,10 +152,11 @@ cudaError_t launch_find_centres(const void* frames, int dtype, int64_t n, int H,
                                 double radius, int iterations, float2* out, cudaStream_t st);
 
 // Two-stage indexing (Section 4.3): per-pixel FP64 sums over frames (accumulate: add onto
-// out), and the mask of kept pixels from the sums (scratch: H * W bytes).
-size_t frame_sum_scratch_bytes(int dtype, int64_t n, int H, int W, int num_sms);
+// out), and the mask of kept pixels from the sums (scratch: H * W bytes).  groups: of frames summed
+// apart (scratch [groups][H][W] when more than one); few: as many as fill the GPU pixel by pixel.
+int frame_sum_groups(int dtype, int64_t n, int H, int W, int num_sms, bool few);
 cudaError_t launch_frame_sum(const void* frames, int dtype, int64_t n, int H, int W, int accumulate, double* out,
-                             double* scratch, int num_sms, cudaStream_t st);
+                             double* scratch, int groups, int num_sms, cudaStream_t st);
 cudaError_t launch_matrix_mask(const double* sum, int H, int W, double thr_n, int n_open, int n_dilate,
                                uint8_t* mask, uint8_t* scratch, int num_sms, cudaStream_t st);
 
