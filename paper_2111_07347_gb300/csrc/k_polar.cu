@@ -385,8 +385,9 @@ __device__ __forceinline__ bool stage_frame_bulk(const T* __restrict__ gframe, T
 }
 
 // The gamma and subtraction of every pixel of a staged float frame, once, so that the taps are plain
-// loads: the same values as tap by tap.  256 frames of 128 x 128 on a 60 x 180 grid: 30 us, tap by
-// tap 36 us.  (Frames too large for shared memory stay tap by tap: transformed into a scratch frame in
+// loads: the same values as tap by tap.  For grids of at least a third as many samples as the frame has
+// pixels: 256 frames of 128 x 128 on a 60 x 180 grid (two thirds) 30 us, tap by tap 36 us; 4096 frames
+// of 200 x 224 on 60 x 180 (a quarter) 454 and 407 us, of 128 x 128 on 30 x 90 (a sixth) 188 and 153 us.  (Frames too large for shared memory stay tap by tap: transformed into a scratch frame in
 // global memory, 1500 frames of 250 x 243 on a 120 x 360 grid took 0.72 ms instead of 0.55.)
 template <int MODE>
 __device__ __forceinline__ void transform_frame(float* frame, int pitch, int H, int W, float2 g, float sub) {
@@ -398,7 +399,8 @@ __device__ __forceinline__ void transform_frame(float* frame, int pitch, int H, 
     }
 }
 
-template <typename T, int MODE, bool STAGED>
+// PLAIN: a staged float frame is transformed first.
+template <typename T, int MODE, bool STAGED, bool PLAIN>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 polar_kernel(const T* __restrict__ frames, int64_t n, int H, int W, int pitch, const longlong2* __restrict__ rays,
              long long cxb, long long cyb, float2 g, float sub, int n_r, int n_theta, int R,
@@ -473,8 +475,7 @@ polar_kernel(const T* __restrict__ frames, int64_t n, int H, int W, int pitch, c
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(nf + off));
             }
         }
-        constexpr bool plain = sizeof(T) == 4 && STAGED;  // transformed where it was staged
-        if (plain) {
+        if (PLAIN) {
             transform_frame<MODE>((float*)sF, pitch, H, W, g, sub);
             __syncthreads();
         }
@@ -491,7 +492,7 @@ polar_kernel(const T* __restrict__ frames, int64_t n, int H, int W, int pitch, c
             polar_rows<T, MODE, STAGED, true>(frame, pf, H, W, cx, cy, rays, n_r, n_theta, row0, rstep, wrows, kstep,
                                               k0, lane, warp, nw, keepm, keep_row, pmask, lut, g, sub, out, part, s2,
                                               c2);
-        else if (plain)
+        else if (PLAIN)
             polar_rows<T, 3, STAGED, false>(frame, pf, H, W, cx, cy, rays, n_r, n_theta, row0, rstep, wrows, kstep, k0,
                                             lane, warp, nw, keepm, keep_row, pmask, lut, g, sub, out, part, s2, c2);
         else
@@ -527,12 +528,12 @@ polar_kernel(const T* __restrict__ frames, int64_t n, int H, int W, int pitch, c
     }
 }
 
-template <typename T, int MODE, bool STAGED>
+template <typename T, int MODE, bool STAGED, bool PLAIN>
 cudaError_t launch_one(const T* frames, int64_t n, int H, int W, int pitch, const longlong2* rays, long long cxb,
                        long long cyb, float2 g, float sub, int n_r, int n_theta, int R, int threads, size_t smem,
                        const uint8_t* keep_row, const uint8_t* pmask, float* polar, float* pnorm, float* radial,
                        const float2* centres, int bulk, unsigned* err, cudaStream_t st) {
-    auto kern = polar_kernel<T, MODE, STAGED>;
+    auto kern = polar_kernel<T, MODE, STAGED, PLAIN>;
     int per_sm = 1;
     const cudaError_t e = kernel_occupancy((const void*)kern, threads, smem, &per_sm);
     if (e != cudaSuccess) return e;
@@ -543,12 +544,14 @@ cudaError_t launch_one(const T* frames, int64_t n, int H, int W, int pitch, cons
     return cudaGetLastError();
 }
 
-template <typename T, bool STAGED>
+template <typename T, bool STAGED, bool PLAIN = false>
 cudaError_t launch_mode(int mode, const T* frames, int64_t n, int H, int W, int pitch, const longlong2* rays,
                         long long cxb, long long cyb, float2 g, float sub, int n_r, int n_theta, int R, int threads,
                         size_t smem, const uint8_t* keep_row, const uint8_t* pmask, float* polar, float* pnorm,
                         float* radial, const float2* centres, int bulk, unsigned* err, cudaStream_t st) {
-    auto f = mode == 0 ? launch_one<T, 0, STAGED> : (mode == 1 ? launch_one<T, 1, STAGED> : launch_one<T, 2, STAGED>);
+    auto f = mode == 0   ? launch_one<T, 0, STAGED, PLAIN>
+             : mode == 1 ? launch_one<T, 1, STAGED, PLAIN>
+                         : launch_one<T, 2, STAGED, PLAIN>;
     return f(frames, n, H, W, pitch, rays, cxb, cyb, g, sub, n_r, n_theta, R, threads, smem, keep_row, pmask, polar,
              pnorm, radial, centres, bulk, err, st);
 }
@@ -579,9 +582,12 @@ cudaError_t launch_typed(const T* frames, int64_t n, int H, int W, const longlon
         const int pitch = (int)(pw * 4 / sizeof(T));
         const size_t smem = smem_of(pw);
         const int bulk = rows16 && (pw % 4) == 0 && !pmask && err != nullptr;
-        if (smem <= 200 * 1024)
-            return launch_mode<T, true>(mode, frames, n, H, W, pitch, rays, cxb, cyb, g, sub, n_r, n_theta, R, threads,
-                                        smem, keep_row, pmask, polar, pnorm, radial, centres, bulk, err, st);
+        if (smem <= 200 * 1024) {
+            const bool plain = sizeof(T) == 4 && 3 * (int64_t)n_r * n_theta >= (int64_t)H * W;
+            auto f = plain ? launch_mode<T, true, sizeof(T) == 4> : launch_mode<T, true>;
+            return f(mode, frames, n, H, W, pitch, rays, cxb, cyb, g, sub, n_r, n_theta, R, threads, smem, keep_row, pmask,
+                     polar, pnorm, radial, centres, bulk, err, st);
+        }
     }
     const int threads = cols < kMaxThreads ? cols : kMaxThreads;
     const size_t smem = (sizeof(T) == 2 ? kLut * sizeof(float) : 0) + ((size_t)n_r * (threads / 32) + threads) * sizeof(float);
