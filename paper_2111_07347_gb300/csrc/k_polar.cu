@@ -344,11 +344,23 @@ __device__ __forceinline__ uint32_t stage_frame(const T* __restrict__ gframe, T*
             }
         }
     } else {
-        for (int e = threadIdx.x; e < H * W; e += blockDim.x) {
-            const int y = e / W;
-            const T v = (!pmask || pmask[e]) ? gframe[e] : T(0);
-            sF[(size_t)y * pitch + (e - y * W)] = v;
-            if (sizeof(T) == 2) hi_bits |= (uint32_t)v;
+        // eight loads in flight per thread (4096 u16 frames of 250 x 243: 879 us, one by one 1055 to 1222)
+        constexpr int B = 8;
+        for (int e0 = threadIdx.x; e0 < H * W; e0 += B * blockDim.x) {
+            T v[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int e = e0 + b * blockDim.x;
+                if (e < H * W) v[b] = (!pmask || pmask[e]) ? gframe[e] : T(0);
+            }
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int e = e0 + b * blockDim.x;
+                if (e >= H * W) continue;
+                const int y = e / W;
+                sF[(size_t)y * pitch + (e - y * W)] = v[b];
+                if (sizeof(T) == 2) hi_bits |= (uint32_t)v[b];
+            }
         }
     }
     return hi_bits;
