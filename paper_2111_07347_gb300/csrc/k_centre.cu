@@ -3,14 +3,52 @@
 // Per pattern, the intensity-weighted centre of mass of the pixels within `radius` of the
 // current estimate, repeated `iterations` times from the starting centre.
 //
-// One warp per pattern visits the disc's bounding box row by row in FP64 with explicitly rounded
-// operations (no fused multiply-adds), so the sums, and hence the centres, are the same bit
-// for bit as a plain double-precision loop in the same order.  The work is a few
-// hundred pixels per pattern; the frames' other pixels are not read.
+// The disc's bounding box is visited row by row in FP64 with explicitly rounded operations (no fused
+// multiply-adds), so the sums, and hence the centres, are the same bit for bit as a plain
+// double-precision loop in the same order.  The work is a few hundred pixels per pattern; the
+// frames' other pixels are not read.  A thread per pattern takes a time that depends on the disc
+// alone until the patterns fill the GPU, a warp per pattern is faster for few patterns or (u16) large
+// discs: launch_find_centres.
 #include "tm_internal.h"
 
 namespace tmgb {
 namespace {
+
+// A thread per pattern: a plain loop.
+template <typename T>
+__global__ void find_centres_thread_kernel(const T* __restrict__ frames, int64_t n, int H, int W, double cx0, double cy0,
+                                    double radius, int iterations, float2* __restrict__ out) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const T* f = frames + (size_t)p * H * W;
+    const double r2 = __dmul_rn(radius, radius);
+    double cx = cx0, cy = cy0;
+    for (int it = 0; it < iterations; ++it) {
+        const int y_lo = max(0, (int)ceil(__dsub_rn(cy, radius)));
+        const int y_hi = min(H - 1, (int)floor(__dadd_rn(cy, radius)));
+        const int x_lo = max(0, (int)ceil(__dsub_rn(cx, radius)));
+        const int x_hi = min(W - 1, (int)floor(__dadd_rn(cx, radius)));
+        double s0 = 0.0, sx = 0.0, sy = 0.0;
+        for (int y = y_lo; y <= y_hi; ++y) {
+            const double dy = __dsub_rn((double)y, cy);
+            const double dy2 = __dmul_rn(dy, dy);
+            for (int x = x_lo; x <= x_hi; ++x) {
+                const double dx = __dsub_rn((double)x, cx);
+                if (__dadd_rn(__dmul_rn(dx, dx), dy2) <= r2) {
+                    const double v = (double)__ldg(f + (size_t)y * W + x);
+                    s0 = __dadd_rn(s0, v);
+                    sx = __dadd_rn(sx, __dmul_rn((double)x, v));
+                    sy = __dadd_rn(sy, __dmul_rn((double)y, v));
+                }
+            }
+        }
+        if (s0 > 0.0) {
+            cx = __ddiv_rn(sx, s0);
+            cy = __ddiv_rn(sy, s0);
+        }
+    }
+    out[p] = make_float2((float)cx, (float)cy);
+}
 
 // One warp per pattern: the lanes take 32 pixels of the disc's box in row order, test them and form
 // their terms (v, x v, y v; 0 outside the disc, which adds nothing), and lanes 0, 1, 2 add the three
@@ -120,9 +158,26 @@ cudaError_t launch_find_centres(const void* frames, int dtype, int64_t n, int H,
     // exact in any order while pixels x value x coordinate stays below 2^53
     const double side = 2.0 * radius + 1.0;
     const double pixels = (side < W ? side : W) * (side < H ? side : H);
-    if (dtype == TM_DTYPE_U16 && pixels * 65535.0 * (W > H ? W : H) < 9.0e15 && pixels < 2.0e9) {
-        find_centres_u16_kernel<<<(unsigned)grid, threads, 0, st>>>((const uint16_t*)frames, n, H, W, cx0, cy0,
-                                                                            radius, iterations, out);
+    const bool exact = dtype == TM_DTYPE_U16 && pixels * 65535.0 * (W > H ? W : H) < 9.0e15 && pixels < 2.0e9;
+    // A warp's time grows with the patterns and its steps of 32 pixels, a thread's with the pixels alone
+    // (up to about 20000 patterns).  256 x 256 frames, warp / thread us: exact sums, 16384 patterns,
+    // radius 1 109 / 14, radius 3 156 / 51, radius 6 203 / 191; f32, 4096 patterns, radius 1 55 / 14,
+    // radius 3 90 / 51, radius 6 185 / 191, radius 20 1620 / 2015; 16384, radius 6 718 / 191, 20 6495 / 2100.
+    const double steps = ceil(pixels / 32.0);
+    const bool warps = exact ? n <= 96.0 * pixels || pixels >= 400.0 : n * (steps + 1.0) <= 150.0 * pixels;
+    if (!warps) {
+        const unsigned blocks = (unsigned)((n + threads - 1) / threads);
+        if (dtype == TM_DTYPE_U16)
+            find_centres_thread_kernel<uint16_t><<<blocks, threads, 0, st>>>((const uint16_t*)frames, n, H, W, cx0, cy0,
+                                                                             radius, iterations, out);
+        else
+            find_centres_thread_kernel<float><<<blocks, threads, 0, st>>>((const float*)frames, n, H, W, cx0, cy0, radius,
+                                                                          iterations, out);
+        return cudaGetLastError();
+    }
+    if (exact) {
+        find_centres_u16_kernel<<<(unsigned)grid, threads, 0, st>>>((const uint16_t*)frames, n, H, W, cx0, cy0, radius,
+                                                                    iterations, out);
         return cudaGetLastError();
     }
     if (dtype == TM_DTYPE_U16)
