@@ -510,11 +510,25 @@ size_t gauss_cols_smem(int H, int r1, int r2, int dog) {
 
 int gauss_padded_taps(int r) { return padded_taps(r); }
 
-// The whole of it in one pass; false when the frames' rolling rows do not fit shared memory.
-bool gauss_stream_supported(int W, int r1, int r2, int rb, bool dog, bool blur) {
+// Whether the whole of it takes one pass: where the frames' rolling rows fit shared memory and the frames
+// are large enough.  A band repeats the filters' reach at its ends, and a narrow or short frame leaves
+// warps of the row filters and bands idle.  One pass against the separate ones, us, u16:
+//   sigma 1 / 4, blur 1 (reach 20): 100 x 100, 1 / 4096 frames 30 / 974 against 31 / 1281;
+//     256 x 256 29 / 2780 against 51 / 5783; 512 x 64 24 / 3630 against 84 / 7557;
+//     32 x 32 25 / 355 against 21 / 247; without blur, 1 frame, 100 x 100 20 against 19, 64 x 512 29
+//     against 19.
+//   sigma 2 / 10, blur 2 (reach 48): 256 x 256 54 / 5970 against 56 / 7280; 144 x 200 52 / 3659
+//     against 41 / 3394.
+//   a blur alone: sigma 1 (reach 4) 256 x 256 15 / 1130 against 21 / 1615, 100 x 100 15 / 471 against
+//     14 / 407; sigma 3 (reach 12) 256 x 256, 16 frames 31 against 27, 300 x 500, 128 frames 225
+//     against 156.
+bool gauss_stream_supported(int H, int W, int r1, int r2, int rb, bool dog, bool blur) {
     StreamShape s;
     int pitch;
-    return (dog || blur) && stream_shape(W, r1, r2, rb, dog, blur, &s, &pitch);
+    if (!(dog || blur) || !stream_shape(W, r1, r2, rb, dog, blur, &s, &pitch)) return false;
+    if (!dog) return rb <= 4 && H >= 144 && W >= 144;
+    const int rows = std::max(blur ? 96 : 112, 5 * (s.R + s.rb));
+    return H >= rows && W >= 64 && (int64_t)H * W >= (int64_t)rows * 96;
 }
 
 namespace {

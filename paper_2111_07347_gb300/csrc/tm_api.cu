@@ -1388,7 +1388,7 @@ int tm_preprocess(tm_ctx* ctx, const tm_preprocess_params* pp, const void* frame
     const char *ib = (const char*)frames_dev, *ob = (const char*)out_dev;
     const size_t in_bytes = (size_t)n * H * W * (dtype == TM_DTYPE_U16 ? 2 : 4);
     const bool apart = ob + img <= ib || ib + in_bytes <= ob;
-    const bool stream_pass = apart && tmgb::gauss_stream_supported(W, r_min, r_max, r_blur, dog, blur);
+    const bool stream_pass = apart && tmgb::gauss_stream_supported(H, W, r_min, r_max, r_blur, dog, blur);
     if (!rc && !stream_pass) rc = workspace(ctx, st, "pre_t1", img, (void**)&t1);
     if (!rc && !stream_pass && dog) rc = workspace(ctx, st, "pre_t2", img, (void**)&t2);
     if (rc) return rc;

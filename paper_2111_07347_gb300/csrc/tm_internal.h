@@ -128,7 +128,7 @@ cudaError_t launch_refine(const RefineCall& c, int num_sms, cudaStream_t st);
 size_t gauss_cols_smem(int H, int r1, int r2, int dog);
 int gauss_padded_taps(int r);               // weights per filter: 2 r + 1 rounded up, zero-padded
 // All passes in one kernel (w1, w2: the difference's filters; wb: the blur's), where it is supported.
-bool gauss_stream_supported(int W, int r1, int r2, int rb, bool dog, bool blur);
+bool gauss_stream_supported(int H, int W, int r1, int r2, int rb, bool dog, bool blur);
 cudaError_t launch_gauss_stream(const void* in, int dtype, int64_t n, int H, int W, const float* w1, int r1,
                                 const float* w2, int r2, const float* wb, int rb, bool dog, bool blur, float* out,
                                 int num_sms, cudaStream_t st);
