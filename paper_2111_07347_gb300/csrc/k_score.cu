@@ -41,18 +41,13 @@ __device__ __forceinline__ float bound_of(uint32_t key) {
     return __half2float(__ushort_as_half((unsigned short)(key & 0x8000u ? key & 0x7fffu : ~key)));
 }
 
-// Results' order as integers: larger is better, -0 ties with 0, and a score that is not a number (an
-// infinite correlation over an infinite norm) is below every number.  kNoKey, read back as a score, is
-// NaN: it compares as no threshold.
-__device__ __forceinline__ unsigned long long order_key(unsigned hi, int k) {
-    return ((unsigned long long)hi << 32) | (0xffffffffu - (unsigned)k);
-}
+// Results' order as integers: larger is better; none is below every template's.  A score that is not a
+// number (an infinite correlation over an infinite norm) ranks below every number: it is -inf here and
+// in the warps' lists, and written out as NaN.
 __device__ __forceinline__ unsigned long long rank_key(float q, int k) {
-    return order_key(q == q ? score_key(q + 0.0f) : 1u, k);             // (score_key(-inf) is 0x007fffff)
+    return ((unsigned long long)score_key(q + 0.0f) << 32) | (0xffffffffu - (unsigned)k);   // (-0 ties with 0)
 }
-constexpr unsigned long long kNoKey = 0;
-// The key no score of template k with bound u exceeds.
-__device__ __forceinline__ unsigned long long bound_rank(float u, int k) { return order_key(score_key(u + 0.0f), k); }
+constexpr unsigned long long kNoKey = 0x007fffffull << 32;              // score -inf, no template
 __device__ __forceinline__ float rank_score(unsigned long long key) { return key_score((unsigned)(key >> 32)); }
 __device__ __forceinline__ unsigned long long warp_min(unsigned long long v) {
     const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(v >> 32));
@@ -219,7 +214,7 @@ score_kernel(const ScoreCall c) {
             float thr_c = -FLT_MAX;
             if (thr > -INFINITY && d > 0.0f) {
                 const float t = thr * d;
-                if (fabsf(t) <= FLT_MAX) thr_c = t - fabsf(t) * 1e-6f;   // (an infinite norm: every template is resolved)
+                thr_c = fmaxf(t - fabsf(t) * 1e-6f, -FLT_MAX);   // (an infinite norm, NaN: every template is resolved)
             }
             int s = 0;
             bool resolved = false;
@@ -230,13 +225,12 @@ score_kernel(const ScoreCall c) {
             float q;
             if (d > 0.0f) q = __fdiv_rn(best, d);
             else { q = 0.0f; s = 0; }
-            if (s >= S) s = 0;                              // (no shift's sum is a number)
-            const unsigned long long key = rank_key(q, k);
+            if (q != q) q = -INFINITY;
             if (lane == 0) {
                 const int cnt_w = lcnt[warp];
-                if (cnt_w < N || key > rank_key(wq[N - 1], wk[N - 1])) {
+                if (cnt_w < N || better(q, k, wq[N - 1], wk[N - 1])) {
                     int i = cnt_w < N ? cnt_w : N - 1;
-                    while (i > 0 && key > rank_key(wq[i - 1], wk[i - 1])) {
+                    while (i > 0 && better(q, k, wq[i - 1], wk[i - 1])) {
                         wq[i] = wq[i - 1]; wk[i] = wk[i - 1]; ws[i] = ws[i - 1];
                         --i;
                     }
@@ -245,7 +239,7 @@ score_kernel(const ScoreCall c) {
                 }
             }
             __syncwarp();
-            return key;
+            return rank_key(q, k);
         };
         // a key into the pool: in place of the smallest while it is larger (warp-collective)
         auto pool_add = [&](unsigned long long key) {
@@ -357,7 +351,7 @@ score_kernel(const ScoreCall c) {
                     const unsigned long long thr = *(volatile unsigned long long*)&s_thr;
                     bool in = !(u_l < rank_score(thr));
                     if (in) meta_l = __ldg(c.order + k0 + lane);
-                    in = in && takes_part(meta_l.w) && bound_rank(u_l, meta_l.w) > thr;
+                    in = in && takes_part(meta_l.w) && rank_key(u_l, meta_l.w) > thr;
                     uint32_t seeded = 0;
                     for (int i = lane; i < nwarps * wseeds; i += 32) {
                         const int sd = s_seed[i];
@@ -393,7 +387,7 @@ score_kernel(const ScoreCall c) {
                         bit = __ffs(m) - 1;
                         fetch();
                     }
-                    if (urow && bound_rank(u_c, cur.w) < *(volatile unsigned long long*)&s_thr) continue;
+                    if (urow && rank_key(u_c, cur.w) < *(volatile unsigned long long*)&s_thr) continue;
                     const unsigned long long key = score_one(cur.w, cur, mine_c);
                     if (key > *(volatile unsigned long long*)&s_thr) pool_add(key);
                 }
@@ -415,9 +409,9 @@ score_kernel(const ScoreCall c) {
             if (rank >= N) continue;
             tm_hit h;
             h.template_index = k;
-            h.shift = ls[i];
-            h.score = q;
-            h.angle_deg = (float)ls[i] * (360.0f / (float)n_theta);
+            h.shift = ls[i] < n_theta ? ls[i] : 0;          // (no shift's sum is a number)
+            h.score = q == -INFINITY ? nanf("") : q;
+            h.angle_deg = (float)h.shift * (360.0f / (float)n_theta);
             h.mirror = (L.mirror && k >= L.K0) ? 1 : 0;
             out[rank] = h;
         }
