@@ -344,23 +344,14 @@ __device__ __forceinline__ uint32_t stage_frame(const T* __restrict__ gframe, T*
             }
         }
     } else {
-        // eight loads in flight per thread (4096 u16 frames of 250 x 243: 879 us, one by one 1055 to 1222)
-        constexpr int B = 8;
-        for (int e0 = threadIdx.x; e0 < H * W; e0 += B * blockDim.x) {
-            T v[B];
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int e = e0 + b * blockDim.x;
-                if (e < H * W) v[b] = (!pmask || pmask[e]) ? gframe[e] : T(0);
-            }
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int e = e0 + b * blockDim.x;
-                if (e >= H * W) continue;
-                const int y = e / W;
-                sF[(size_t)y * pitch + (e - y * W)] = v[b];
-                if (sizeof(T) == 2) hi_bits |= (uint32_t)v[b];
-            }
+        // (unrolled, so that loads overlap: 4096 u16 frames of 250 x 243 987 us, one by one 1055 to 1222;
+        // eight by hand 871, but 11 to 14 % slower on single frames)
+#pragma unroll 4
+        for (int e = threadIdx.x; e < H * W; e += blockDim.x) {
+            const int y = e / W;
+            const T v = (!pmask || pmask[e]) ? gframe[e] : T(0);
+            sF[(size_t)y * pitch + (e - y * W)] = v;
+            if (sizeof(T) == 2) hi_bits |= (uint32_t)v;
         }
     }
     return hi_bits;
@@ -411,13 +402,15 @@ __device__ __forceinline__ void transform_frame(float* frame, int pitch, int H, 
     }
 }
 
-// PLAIN: a staged float frame is transformed first.
-template <typename T, int MODE, bool STAGED, bool PLAIN>
+// PLAIN: a staged float frame is transformed first.  BULK: frames are staged by bulk copies.
+// (Both at compile time: with the two ways of staging in one kernel, changes to the scalar one moved the
+// bulk one's time by 5 %.  4096 u16 frames of 256 x 256 on 100 x 360: 494 us, in one kernel 526 to 539.)
+template <typename T, int MODE, bool STAGED, bool PLAIN, bool BULK>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 polar_kernel(const T* __restrict__ frames, int64_t n, int H, int W, int pitch, const longlong2* __restrict__ rays,
              long long cxb, long long cyb, float2 g, float sub, int n_r, int n_theta, int R,
              const uint8_t* __restrict__ keep_row, const uint8_t* __restrict__ pmask, float* __restrict__ polar,
-             float* __restrict__ pnorm, float* __restrict__ radial, const float2* __restrict__ centres, int bulk,
+             float* __restrict__ pnorm, float* __restrict__ radial, const float2* __restrict__ centres,
              unsigned* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int cols = blockDim.x / R;                     // threads per row group (multiple of 32)
@@ -443,7 +436,7 @@ polar_kernel(const T* __restrict__ frames, int64_t n, int H, int W, int pitch, c
     float* part = lut + (kHasLut ? kLut : 0);                           // [n_r][nw]
     float* red = part + (size_t)n_r * nw;                               // [blockDim]
     uint64_t* bar = (uint64_t*)(((uintptr_t)(red + blockDim.x) + 7) & ~(uintptr_t)7);   // bulk staging
-    if (STAGED && bulk && threadIdx.x == 0) mbar_init1(bar);
+    if (BULK && threadIdx.x == 0) mbar_init1(bar);
     uint32_t staged = 0;                                                // frames staged by bulk copies
     if (kHasLut) {
         for (int i = threadIdx.x; i < kLut; i += blockDim.x) {
@@ -460,7 +453,7 @@ polar_kernel(const T* __restrict__ frames, int64_t n, int H, int W, int pitch, c
         if (STAGED) {
             __syncthreads();                             // previous pattern's reads are done
             uint32_t hi_bits = 0;
-            if (bulk) {
+            if (BULK) {
                 if (!stage_frame_bulk<T>(gframe, sF, H, W, pitch, bar, staged & 1u, hi_bits)) {
                     // the copy did not land in time: report it, let it finish (bounded), stop
                     if (threadIdx.x == 0) {
@@ -540,32 +533,32 @@ polar_kernel(const T* __restrict__ frames, int64_t n, int H, int W, int pitch, c
     }
 }
 
-template <typename T, int MODE, bool STAGED, bool PLAIN>
+template <typename T, int MODE, bool STAGED, bool PLAIN, bool BULK>
 cudaError_t launch_one(const T* frames, int64_t n, int H, int W, int pitch, const longlong2* rays, long long cxb,
                        long long cyb, float2 g, float sub, int n_r, int n_theta, int R, int threads, size_t smem,
                        const uint8_t* keep_row, const uint8_t* pmask, float* polar, float* pnorm, float* radial,
-                       const float2* centres, int bulk, unsigned* err, cudaStream_t st) {
-    auto kern = polar_kernel<T, MODE, STAGED, PLAIN>;
+                       const float2* centres, unsigned* err, cudaStream_t st) {
+    auto kern = polar_kernel<T, MODE, STAGED, PLAIN, BULK>;
     int per_sm = 1;
     const cudaError_t e = kernel_occupancy((const void*)kern, threads, smem, &per_sm);
     if (e != cudaSuccess) return e;
     int64_t grid = (int64_t)device_sms() * (per_sm > 0 ? per_sm : 1);
     if (grid > n) grid = n;
     kern<<<(int)grid, threads, smem, st>>>(frames, n, H, W, pitch, rays, cxb, cyb, g, sub, n_r, n_theta, R, keep_row,
-                                           pmask, polar, pnorm, radial, centres, bulk, err);
+                                           pmask, polar, pnorm, radial, centres, err);
     return cudaGetLastError();
 }
 
-template <typename T, bool STAGED, bool PLAIN = false>
+template <typename T, bool STAGED, bool PLAIN = false, bool BULK = false>
 cudaError_t launch_mode(int mode, const T* frames, int64_t n, int H, int W, int pitch, const longlong2* rays,
                         long long cxb, long long cyb, float2 g, float sub, int n_r, int n_theta, int R, int threads,
                         size_t smem, const uint8_t* keep_row, const uint8_t* pmask, float* polar, float* pnorm,
-                        float* radial, const float2* centres, int bulk, unsigned* err, cudaStream_t st) {
-    auto f = mode == 0   ? launch_one<T, 0, STAGED, PLAIN>
-             : mode == 1 ? launch_one<T, 1, STAGED, PLAIN>
-                         : launch_one<T, 2, STAGED, PLAIN>;
+                        float* radial, const float2* centres, unsigned* err, cudaStream_t st) {
+    auto f = mode == 0   ? launch_one<T, 0, STAGED, PLAIN, BULK>
+             : mode == 1 ? launch_one<T, 1, STAGED, PLAIN, BULK>
+                         : launch_one<T, 2, STAGED, PLAIN, BULK>;
     return f(frames, n, H, W, pitch, rays, cxb, cyb, g, sub, n_r, n_theta, R, threads, smem, keep_row, pmask, polar,
-             pnorm, radial, centres, bulk, err, st);
+             pnorm, radial, centres, err, st);
 }
 
 template <typename T>
@@ -593,19 +586,21 @@ cudaError_t launch_typed(const T* frames, int64_t n, int H, int W, const longlon
         if (smem_of(pw) > 200 * 1024) pw = words | 1;
         const int pitch = (int)(pw * 4 / sizeof(T));
         const size_t smem = smem_of(pw);
-        const int bulk = rows16 && (pw % 4) == 0 && !pmask && err != nullptr;
+        const bool bulk = rows16 && (pw % 4) == 0 && !pmask && err != nullptr;
         if (smem <= 200 * 1024) {
             const bool plain = sizeof(T) == 4 && 3 * (int64_t)n_r * n_theta >= (int64_t)H * W;
-            auto f = plain ? launch_mode<T, true, sizeof(T) == 4> : launch_mode<T, true>;
+            constexpr bool F = sizeof(T) == 4;
+            auto f = plain ? (bulk ? launch_mode<T, true, F, true> : launch_mode<T, true, F, false>)
+                           : (bulk ? launch_mode<T, true, false, true> : launch_mode<T, true, false, false>);
             return f(mode, frames, n, H, W, pitch, rays, cxb, cyb, g, sub, n_r, n_theta, R, threads, smem, keep_row, pmask,
-                     polar, pnorm, radial, centres, bulk, err, st);
+                     polar, pnorm, radial, centres, err, st);
         }
     }
     const int threads = cols < kMaxThreads ? cols : kMaxThreads;
     const size_t smem = (sizeof(T) == 2 ? kLut * sizeof(float) : 0) + ((size_t)n_r * (threads / 32) + threads) * sizeof(float);
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
     return launch_mode<T, false>(mode, frames, n, H, W, W, rays, cxb, cyb, g, sub, n_r, n_theta, 1, threads, smem,
-                                 keep_row, pmask, polar, pnorm, radial, centres, 0, err, st);
+                                 keep_row, pmask, polar, pnorm, radial, centres, err, st);
 }
 
 }  // namespace
