@@ -63,7 +63,9 @@ __device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
 // Largest block: 64 registers a thread hold up to 12 accumulators a lane, else 128.
 constexpr int max_threads(int nb_max) { return nb_max <= 12 ? 1024 : 512; }
 
-template <int NBMAX, int LAYOUT>
+// BOUNDS: behind bounds (c.u), or the templates of the mask.  At compile time: together in one kernel,
+// the registers of each cost the other up to 7 %.
+template <int NBMAX, int LAYOUT, bool BOUNDS>
 __global__ void __launch_bounds__(max_threads(NBMAX), 1)
 score_kernel(const ScoreCall c) {
     extern __shared__ __align__(16) float smem[];
@@ -92,8 +94,11 @@ score_kernel(const ScoreCall c) {
     int* ws = ls + warp * N;
     unsigned long long work = 0;                            // multiply-adds of this warp (lane 0)
     const int wseeds = max(1, c.seeds / nwarps);            // seeds per warp
-    // without bounds, items of 8 templates while the words alone would not occupy the warps
-    const int part = !c.u && L.words < 8 * nwarps ? 2 : 0;
+    // items of 8 templates while the words alone would not occupy the warps (with bounds, which leave
+    // few templates of most words, only in the large blocks of few patterns or long rows and up to 2048
+    // templates: 64 patterns against 600 templates that the bounds cannot tell apart 279 us, by words
+    // 328; 1024 against 1000 of them 2064 and 2282)
+    const int part = (BOUNDS ? nwarps >= 16 && L.words < 64 : L.words < 8 * nwarps) ? 2 : 0;
     auto part_mask = [&](int w) -> uint32_t { return part ? 0xffu << (8 * (w & 3)) : 0xffffffffu; };
 
     for (;;) {
@@ -112,8 +117,8 @@ score_kernel(const ScoreCall c) {
         const float* src = c.polar + (size_t)p * c.n_r * n_theta;
         const float pn = __ldg(c.pnorm + p);
         const uint32_t* mrow = c.mask ? c.mask + (size_t)p * L.words : nullptr;
-        const unsigned short* urow = c.u ? c.u + (size_t)p * L.words * 32 : nullptr;
-        const unsigned short* wrow = c.u ? c.wmax + (size_t)p * L.words : nullptr;
+        const unsigned short* urow = BOUNDS ? c.u + (size_t)p * L.words * 32 : nullptr;
+        const unsigned short* wrow = BOUNDS ? c.wmax + (size_t)p * L.words : nullptr;
 
         // ---- the library's polar rows
         if (bulk) {
@@ -148,7 +153,7 @@ score_kernel(const ScoreCall c) {
                 const char* a = reinterpret_cast<const char*>(nsrc + (size_t)__ldg(L.radii + r0) * n_theta) + 128 * l;
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
             }
-            if (urow && threadIdx.x * 64 < L.words)
+            if (BOUNDS && threadIdx.x * 64 < L.words)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(wrow + (size_t)gridDim.x * L.words + threadIdx.x * 64));
         }
         // whether the template at a position takes part (bounds: positions are in `order`)
@@ -162,7 +167,7 @@ score_kernel(const ScoreCall c) {
         };
         // ---- seeds: of the warp's words (w = warp mod nwarps), those of highest maximum
         int seed_l = -1;                                    // lane i < wseeds: position of the warp's i-th seed
-        if (urow) {
+        if (BOUNDS) {
             uint32_t best = 0;                              // lane's best word: maximum << 16 | local index
             for (int i = lane; warp + i * nwarps < L.words; i += 32) {
                 const uint32_t m = __ldg(wrow + warp + i * nwarps);
@@ -265,7 +270,7 @@ score_kernel(const ScoreCall c) {
         };
 
         unsigned long long thr0 = kNoKey;                   // the N-th best of the seeds
-        if (urow) {
+        if (BOUNDS) {
             // the seeds, each one's metadata and spots on their way before the one before is scored
             int4 meta_l = make_int4(0, 0, 0, -1);
             if (seed_l >= 0) meta_l = __ldg(c.order + seed_l);
@@ -325,8 +330,8 @@ score_kernel(const ScoreCall c) {
                 const int w = b + lane;
                 bool in = w < items;
                 if (in)
-                    in = urow ? !(bound_of(__ldg(wrow + w)) < cut0)
-                              : (word_mask(w >> part) & part_mask(w)) != 0u;
+                    in = BOUNDS ? !(bound_of(__ldg(wrow + (w >> part))) < cut0)
+                                : (word_mask(w >> part) & part_mask(w)) != 0u;
                 const unsigned bal = __ballot_sync(0xffffffffu, in);
                 int at = 0;
                 if (lane == 0 && bal) at = atomicAdd(&s_push, __popc(bal));
@@ -344,7 +349,7 @@ score_kernel(const ScoreCall c) {
                 uint32_t m;
                 int4 meta_l = make_int4(0, 0, 0, 0);
                 float u_l = INFINITY;
-                if (urow) {
+                if (BOUNDS) {
                     // the word's templates that take part, not the seeds, that the threshold as it is
                     // now leaves
                     u_l = bound_of(__ldg(urow + k0 + lane));
@@ -355,9 +360,9 @@ score_kernel(const ScoreCall c) {
                     uint32_t seeded = 0;
                     for (int i = lane; i < nwarps * wseeds; i += 32) {
                         const int sd = s_seed[i];
-                        if ((sd >> 5) == w) seeded |= 1u << (sd & 31);
+                        if ((sd >> 5) == (w >> part)) seeded |= 1u << (sd & 31);
                     }
-                    m = __ballot_sync(0xffffffffu, in) & ~__reduce_or_sync(0xffffffffu, seeded);
+                    m = __ballot_sync(0xffffffffu, in) & ~__reduce_or_sync(0xffffffffu, seeded) & part_mask(w);
                 } else {
                     m = word_mask(w >> part) & part_mask(w);
                     if ((m >> lane) & 1u) {
@@ -387,7 +392,7 @@ score_kernel(const ScoreCall c) {
                         bit = __ffs(m) - 1;
                         fetch();
                     }
-                    if (urow && rank_key(u_c, cur.w) < *(volatile unsigned long long*)&s_thr) continue;
+                    if (BOUNDS && rank_key(u_c, cur.w) < *(volatile unsigned long long*)&s_thr) continue;
                     const unsigned long long key = score_one(cur.w, cur, mine_c);
                     if (key > *(volatile unsigned long long*)&s_thr) pool_add(key);
                 }
@@ -473,8 +478,8 @@ int block_sizes(int n_rad, int n_theta, int pitch, int top_n, int threads[3]) {
     return n;
 }
 
-template <int NBMAX, int LAYOUT>
-cudaError_t launch_nb(const ScoreCall& c, int num_sms, cudaStream_t st) {
+template <int NBMAX, int LAYOUT, bool BOUNDS>
+cudaError_t launch_sizes(const ScoreCall& c, int num_sms, cudaStream_t st) {
     // Block size: with at most two patterns per SM, as many warps on each as fit; else the smallest
     // block that fills the SM's registers (blocks run their phases out of step).
     int threads = 0, per_sm = 0;
@@ -486,7 +491,7 @@ cudaError_t launch_nb(const ScoreCall& c, int num_sms, cudaStream_t st) {
         const int t = sizes[i];
         int b = 0;
         const size_t sm = score_smem(c.lib.n_rad, c.pitch, c.top_n, t / 32);
-        const cudaError_t e = kernel_occupancy((const void*)score_kernel<NBMAX, LAYOUT>, t, sm, &b);
+        const cudaError_t e = kernel_occupancy((const void*)score_kernel<NBMAX, LAYOUT, BOUNDS>, t, sm, &b);
         if (e != cudaSuccess) return e;
         const int64_t used = std::min<int64_t>(b, share);
         if (b > 0 && used * t > (int64_t)threads * std::min<int64_t>(per_sm, share)) {
@@ -498,8 +503,13 @@ cudaError_t launch_nb(const ScoreCall& c, int num_sms, cudaStream_t st) {
     if (!threads) return cudaErrorInvalidConfiguration;
     int64_t grid = (int64_t)num_sms * per_sm;
     if (grid > c.n) grid = c.n;
-    score_kernel<NBMAX, LAYOUT><<<(int)grid, threads, smem, st>>>(c);
+    score_kernel<NBMAX, LAYOUT, BOUNDS><<<(int)grid, threads, smem, st>>>(c);
     return cudaGetLastError();
+}
+
+template <int NBMAX, int LAYOUT>
+cudaError_t launch_nb(const ScoreCall& c, int num_sms, cudaStream_t st) {
+    return c.u ? launch_sizes<NBMAX, LAYOUT, true>(c, num_sms, st) : launch_sizes<NBMAX, LAYOUT, false>(c, num_sms, st);
 }
 
 }  // namespace
