@@ -852,10 +852,21 @@ int ensure_spectra(tm_ctx* ctx, Library* L, const SpectralTables& spec, cudaStre
     return TM_OK;
 }
 
-// A library of less templates is scored whole: the bounds' two launches and their latency cost more
-// than the scores they would save (300 templates of 24 spots, 256 patterns: 137 us with bounds, 83 us
-// without).
-constexpr int kBoundTemplates = 512;
+// Whether a call scores every template of a library: the bounds' two launches and their latency cost
+// more than the scores they would save, for few templates, unless these have few spots (the bounds
+// then leave few of them) and the patterns are many.  Bounds / whole, us, 256 x 256 frames:
+//   428 templates of 7 spots: 64 patterns 83 / 73, 256 108 / 120, 8192 1751 / 2714;
+//   348 of 13: 64 107 / 82, 256 157 / 137, 1024 391 / 439; 242 of 7: 256 106 / 95, 1024 267 / 298;
+//   500 of 24: 64 232 / 197, 1024 1246 / 1229; 216 of 34: 64 127 / 98, 8192 4318 / 4121;
+//   100 of 24: 64 130 / 86, 8192 3615 / 2999;
+//   604 of 7: 64 78 / 85, 8192 1799 / 3249; 700 of 24: 64 294 / 262, 8192 11140 / 12319;
+//   806 of 34: 1 117 / 242, 64 264 / 245, 8192 6241 / 11695.
+bool may_bound(const Library* L) {
+    return L->K >= 512 || (L->K >= 200 && (int64_t)L->r.size() <= 16 * L->K);
+}
+bool scored_whole(const Library* L, int64_t n) {
+    return !may_bound(L) || (L->K < 512 && n * L->K < 100000);
+}
 
 size_t bound_order_at(const Library* L) { return ((size_t)L->K * L->bshape.pitch * 2 + 255) & ~(size_t)255; }
 size_t bound_need(const Library* L) {
@@ -1623,7 +1634,7 @@ int tm_load_library(tm_ctx* ctx, const tm_library_desc* desc, int* lib_id) {
     }
     // the bound templates at once, so that the first indexing call need not wait for them; with a budget
     // they are left to a call that uses them, and later loads find the room
-    if (!ctx->budget && L->boundable && L->K >= kBoundTemplates) build_bounds(ctx, L.get(), nullptr);
+    if (!ctx->budget && L->boundable && may_bound(L.get())) build_bounds(ctx, L.get(), nullptr);
     const int id = ctx->next_id++;
     ctx->libs.emplace(id, std::move(L));
     *lib_id = id;
@@ -1894,7 +1905,7 @@ int tmgb::index_patterns_ex(tm_ctx* ctx, const tm_index_params* params, const vo
     Library* bounded[TM_MAX_LIBS];
     for (int i = 0; i < n_libs; ++i) {
         scores = scores && tmgb::score_supported((int)std::max<size_t>(1, libs[i]->radii.size()), n_theta, N);
-        whole[i] = libs[i]->K < kBoundTemplates;
+        whole[i] = scored_whole(libs[i], n);
         bounded[i] = whole[i] ? nullptr : libs[i];
     }
     // (while shapes of the sparse kernel are timed, it serves the call)

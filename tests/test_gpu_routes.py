@@ -132,3 +132,24 @@ def test_refinement_leaves_unwritten_rows_alone():
     ctx.check()
     assert (out[..., 0] >= 0).all()
     ctx.close()
+
+
+@pytest.mark.parametrize("which,step,K,n,launches", [
+    ("hcp", 4.0, 242, 413, 2), ("hcp", 4.0, 242, 414, BOUND_LAUNCHES),     # 100000 pattern-template pairs
+    ("fcc+", 3.0, 216, 600, 2),                                            # 34 spots a template: always whole
+    ("few", 4.0, 199, 1000, 2), ("few", 4.0, 200, 1000, BOUND_LAUNCHES)])
+def test_small_libraries_on_both_sides_of_the_rule(which, step, K, n, launches):
+    if which == "few":
+        ts = synth.random_templates(synth.make_rng(8), K, spots=(4, 12))
+    else:
+        ts = synth.kinematic_library(which.rstrip("+"), step_deg=step,
+                                     **(synth.MULTIPHASE_KINEMATICS if which.endswith("+") else {}))
+    f = _frames(ts, 60, 180, 88).repeat(-(-n // 60), 1, 1)[:n].contiguous()
+    ctx = tmgb.Context(0)
+    lid = ctx.load_library(ts, 100, 180)
+    assert ctx.library_info(lid)["n_templates"] == K
+    hits = tmgb.hits_to_numpy(ctx.index(f, lid, top_n=5))[0]
+    assert ctx.last_stats["launches"] == launches
+    ctx.check()
+    _check(ctx, lid, f, hits, 100, 180, 5)
+    ctx.close()
