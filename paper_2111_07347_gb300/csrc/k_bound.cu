@@ -444,10 +444,14 @@ int bound_stages(int kd) {
 
 }  // namespace
 
-// Six windows, twelve where templates of like weights compete (`fine`).  Bounds and scores together,
-// ms: HCP library with its intensities, 32768 patterns, 6.05 with six and 8.83 with twelve; the same
-// library with unit intensities over a subtracted background, 8192 patterns, 6.04 and 3.48 (six leave
-// four times the scores).
+// Six windows, twelve where templates of like weights compete (`fine`: unit intensities, or 20 and
+// more spots a template).  Twelve cost more to make and leave fewer scores.  The whole call, us, six /
+// twelve, 1024 patterns without pre-filter: 3 spots 567 / 548, with unit intensities 693 / 667; 7 spots
+// 406 / 482, unit 545 / 505; 12 spots (20896 templates) 616 / 672, (5292) 569 / 475; 24 spots 2433 / 2265;
+// 33 spots (6990) 1873 / 1114, (1780) 1449 / 941.  8192 patterns: 3 spots 2415 / 2561, 7 spots 2561 /
+// 3166, unit 2986 / 3261, 33 spots (1780) 8837 / 5275.  64 patterns: 7 spots 100 / 109, unit 159 / 119,
+// 33 spots 354 / 204.  Unit intensities over a subtracted background (two-stage scan, bounds and scores,
+// 8192 patterns): 6040 / 3480.  Between 8 and 20 spots either side wins by up to a sixth.
 bool bound_shape(int n_rad, int n_theta, bool fine, BoundShape* out) {
     if (n_rad < 1 || n_theta < 64) return false;
     BoundShape s;

@@ -10,8 +10,10 @@
 // (divided by |P|), so C is Q directly.  Stage A (G, a GEMM per frequency over the radii) runs
 // before this kernel and leaves G in global memory as BF16, frequency-major:
 //   G[j][p][c][k]  (slot j, pattern p of the batch, c = 0 real / 1 imaginary, template k),
-// slot j < 96 holding m = 2 j and slot j >= 96 holding m = 2 (j - 96) + 1; slots with m > H are not
-// read (their K rows are filled with zeros by the tensor maps' bounds).  Two radix-2 splits quarter
+// slot j < 96 holding m = 2 j and slot j >= 96 holding m = 2 (j - 96) + 1.  Slots with m > H add
+// nothing: their rows of the basis are zero, and where the even and odd slots have a tensor map each
+// they lie outside it and are not read (zero fill); small batches compute and read all slots through
+// one map, their spectra being zero.  Two radix-2 splits quarter
 // the work of the full sum.  With E[s] the even-m part and O[s] the odd-m part of the sum, C[s] = E[s] + O[s]
 // and C[s + H] = E[s] - O[s], so max(C[s], C[s + H]) = E[s] + |O[s]| for s < H.  And with the cosine (real)
 // and sine (imaginary) parts of each, E = Ec + Es, O = Oc + Os, their symmetry about H / 2 gives
@@ -199,6 +201,9 @@ __global__ void __launch_bounds__(kThreads, 1) dense_kernel(const __grid_constan
             bool stop = false, issued = false;
             uint32_t last_bar = 0, last_par = 0;
             for (Unit w(tiles); w.p < c.n && !stop; w.next(), ++tt) {
+                // kept rolled: fully unrolled by nvcc 13.0 it gave wrong sums, and reading the phases, the
+                // blocks' rotation and the descriptors shows no reason (test_gpu_tensor.py compares every
+                // pre-score with the oracle's)
 #pragma unroll 1
                 for (int ch = 0; ch < kParts; ++ch, ++g) {
                     const uint32_t slot = g % kStages, use = g / kStages;
@@ -242,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_kernel(const __grid_constan
             }
         }
     } else if (warp >= kEpiWarp0) {
-        // ================================================================ epilogue (warps 4-11)
+        // ================================================================ epilogue (warps 4-19)
         const int ew = warp - kEpiWarp0;
         const int quad = warp & 3, quarter = ew >> 2;         // TMEM lanes 32 quad.., shift columns by quarter
         const int row = quad * 32 + lane;
