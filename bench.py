@@ -18,7 +18,8 @@ loop; the two-stage masked workflow; preprocessing; template simulation.
 `--impl reference` times the FP64 CPU oracle on the host cores on bounded samples of the
 headline workload (there is no other reference implementation of this paper).
 
-Prints one JSON line (rank 0).
+Prints one JSON line (rank 0); the whole record, with every workload's stages and rooflines,
+goes to stderr.
 """
 from __future__ import annotations
 
@@ -750,6 +751,24 @@ def bench_workload(args, ctx, timer, name, libs_ts, lids, frames_d, frames_np_un
     return rec, res
 
 
+def compact_line(line):
+    """The result line: everything but the per-workload and per-path records, of which it keeps each
+    path's rate, time, launches and agreement (the whole record, some 20 KB, goes to stderr)."""
+    def path_summary(r):
+        if "unsupported" in r:
+            return r
+        agree = ((r.get("top1_vs_oracle") or {}).get("all") or {}).get("rate")
+        return {"patterns_per_s": r["patterns_per_s"], "ms_per_step": r["ms_per_step"],
+                "launches_per_step": r["launches_per_step"], "top1_vs_oracle": agree,
+                "stage_ms": {k: round(v["ms_per_step"], 4) for k, v in r["stages"].items()}}
+
+    out = {k: v for k, v in line.items() if k not in ("workloads", "paths")}
+    out["workloads"] = {wl: {"patterns": rec["patterns"],
+                             "paths": {nm: path_summary(r) for nm, r in rec["paths"].items()}}
+                        for wl, rec in line["workloads"].items()}
+    return out
+
+
 def run_ours(args):
     import torch
     rank, local, world = dist_env()
@@ -912,7 +931,8 @@ def run_ours(args):
         line["template_simulation"] = simulation_bench(ctx, stream)
         del frames_d
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)     # every record
+        print(json.dumps(compact_line(line)), flush=True)
     ctx.close()
     if world > 1:
         torch.distributed.destroy_process_group()
